@@ -20,56 +20,21 @@ namespace {
 // Runs above this many body ADOs keep launches of their own: the work-list kernel reads H from
 // shared memory instead of the constant bank, which costs at the sizes where one run fills the GPU.
 constexpr int64_t kListRunMaxAdos = 200000;
-// Chunks per work item: one per warp (4-warp FP32 body kernel, 2-warp FP64 head kernel), so that a
-// small run spreads over as many CTAs as it has chunks -- at these sizes a launch is latency-bound,
-// and the FP64 head of a large n_states (one ADO per chunk) is the longest chain.
+// Chunks per work item: one per warp of the 4-warp FP32 body kernel, so that a small run spreads over as many
+// CTAs as it has chunks -- at these sizes a launch is latency-bound.
 constexpr int kListCpiBody = 4;
-constexpr int kListCpiHead = 2;
-const char kListTag = 0;          // desc_owner of runs whose descriptor area holds work-list arguments
 
-// The Horner stages of one RK4 step: (input, base, output, coefficient of h).
+// The Horner stages of one RK4 step: input, base, output (horner_c: the coefficient).
 struct HornerStage {
   int zin, y, out;  // 0 = y, 1 = zA, 2 = zB
-  double c;
 };
-constexpr HornerStage kHorner[4] = {{0, 0, 1, 0.25}, {1, 0, 2, 1.0 / 3.0}, {2, 0, 1, 0.5}, {1, 0, 0, 1.0}};
+constexpr HornerStage kHorner[4] = {{0, 0, 1}, {1, 0, 2}, {2, 0, 1}, {1, 0, 0}};
 
 StateView view_of(const heom_run *r, int k) { return k == 0 ? r->y : (k == 1 ? r->zA : r->zB); }
 
 bool list_eligible(const heom_run *r) {
   return r->precision == HEOM_FP32_MIXED && !r->vec && !r->gen && !r->has_field && !r->cplx_h && r->u_split > 0 &&
          r->n_ado - r->u_split <= kListRunMaxAdos;
-}
-
-template <typename CT>
-void fill_args(GroupArgs<CT> &g, const heom_run *r, int st, double h, bool head) {
-  const HornerStage &hs = kHorner[st];
-  std::memset(&g, 0, sizeof(g));
-  g.c = common_for(r, view_of(r, hs.zin), view_of(r, hs.y), view_of(r, hs.out));
-  g.c.u_begin = head ? 0 : r->u_split;
-  g.c.u_end = head ? r->u_split : (int)r->n_ado;
-  g.c.occ_pct = r->sched[head ? 1 : 0].occupancy_pct;
-  g.c.cpw = r->sched[head ? 1 : 0].chunks_per_warp;
-  g.ch = (CT)(hs.c * h);
-  for (int i = 0; i < kMaxStates; ++i) g.term[i] = (i < r->n) ? (CT)r->term[i] : (CT)0;
-  for (int i = 0; i < r->n; ++i)
-    for (int j = 0; j < r->n; ++j) g.H[i * kMaxStates + j] = (CT)r->H[(size_t)i * r->n + j];
-}
-
-// The run's work-list stage arguments for time step h, written into its descriptor area on stream s
-// unless they are there already.
-int ensure_args(heom_run *r, double h, cudaStream_t s, std::vector<GroupRunDesc> &host, size_t k) {
-  if (r->desc_owner == &kListTag && r->desc_dt == h) return HEOM_OK;
-  GroupRunDesc &d = host[k];
-  for (int st = 0; st < 4; ++st) {
-    fill_args(d.body[st], r, st, h, false);
-    fill_args(d.head[st], r, st, h, true);
-  }
-  cudaError_t e = cudaMemcpyAsync(r->desc_dev, &d, sizeof(GroupRunDesc), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return cuda_fail("heom_group_propagate: stage arguments", e);
-  r->desc_owner = &kListTag;
-  r->desc_dt = h;
-  return HEOM_OK;
 }
 
 }  // namespace
@@ -145,12 +110,11 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   }
 
   // work-list arguments of the eligible runs
-  std::vector<GroupRunDesc> host(n_runs);
   std::vector<bool> listed(n_runs);
   for (int i = 0; i < n_runs; ++i) {
     listed[i] = list_eligible(rv[i]) && n_steps[i] > 0;
     if (listed[i]) {
-      const int rc = ensure_args(rv[i], h, gs, host, (size_t)i);
+      const int rc = el_group_args(rv[i], h, gs);
       if (rc != HEOM_OK) {
         cleanup();
         return rc;
@@ -159,6 +123,19 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   }
 
   int rc = HEOM_OK;
+  // small FP64 runs: whole steps in shared launches (resident.cuh), before the others' stages
+  std::vector<bool> done(n_runs, false);
+  if (!capturing(gs)) {
+    std::vector<heom_run *> small;
+    std::vector<int64_t> small_steps;
+    for (int i = 0; i < n_runs; ++i) {
+      done[i] = !listed[i] && n_steps[i] > 0 && rv[i]->precision == HEOM_FP64 && el_small(rv[i]);
+      if (!done[i]) continue;
+      small.push_back(rv[i]);
+      small_steps.push_back(n_steps[i]);
+    }
+    if (!small.empty()) rc = el_propagate(small.data(), (int)small.size(), h, small_steps.data(), obs_stride, gs);
+  }
   // Each size class gets a stream of its own for the whole call (forked from and joined back into the
   // caller's stream): the classes' launch chains run side by side, while the stages of one class
   // follow each other.  A run keeps its class, so its launches stay in order.
@@ -168,7 +145,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   bool single = true;
   int n0 = -1;
   for (int i = 0; i < n_runs && single; ++i) {
-    if (n_steps[i] == 0) continue;
+    if (n_steps[i] == 0 || done[i]) continue;
     if (n0 < 0) n0 = rv[i]->n;
     single = listed[i] && rv[i]->n == n0;
   }
@@ -196,9 +173,11 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   // the work-list launches of one step, rebuilt only when a run's steps end: per class of equal
   // n_states and per batch of at most kListMaxRuns runs, the head and body launch of each stage
   struct Prepared {
-    int n, kind, sm_count;
+    int n, sm_count;
+    bool head;
     cudaStream_t stream;
     ListLaunch L[4];
+    HeadList H;
     std::vector<heom_run *> members;
   };
   std::vector<Prepared> prep;
@@ -214,39 +193,65 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       for (const auto &cl : classes) {
         cudaStream_t cs = gs;
         if ((rc = class_stream(cl.first, &cs)) != HEOM_OK) break;
-        for (size_t b0 = 0; b0 < cl.second.size(); b0 += kListMaxRuns) {
-          const size_t b1 = std::min(cl.second.size(), b0 + (size_t)kListMaxRuns);
-          for (int part = 0; part < 2; ++part) {  // FP64 head, then FP32 body
+        // FP64 heads: Hermitian runs and others take different kernels
+        for (int herm = 0; herm < 2; ++herm) {
+          std::vector<heom_run *> hr;
+          for (int i : cl.second)
+            if ((rv[i]->herm ? 1 : 0) == herm) hr.push_back(rv[i]);
+          for (size_t b0 = 0; b0 < hr.size(); b0 += kListMaxRuns) {
             Prepared p;
             p.n = cl.first;
-            p.kind = part == 0 ? 2 : 1;
-            p.sm_count = rv[cl.second[b0]]->sm_count;
+            p.head = true;
+            p.sm_count = hr[0]->sm_count;
             p.stream = cs;
-            for (int st = 0; st < 4; ++st) {
-              ListLaunch &L = p.L[st];
-              L.nruns = (int)(b1 - b0);
-              L.cpi = part == 0 ? kListCpiHead : kListCpiBody;
-              L.item0[0] = 0;
-              for (size_t q = b0; q < b1; ++q) {
-                const heom_run *r = rv[cl.second[q]];
-                const GroupRunDesc *d = reinterpret_cast<const GroupRunDesc *>(r->desc_dev);
-                const int A = 32 / r->n < 32 ? 32 / r->n : 31;
-                const int64_t ados = part == 0 ? r->u_split : r->n_ado - r->u_split;
-                const int64_t chunks = (ados + A - 1) / A;
-                L.args[q - b0] = part == 0 ? (const void *)&d->head[st] : (const void *)&d->body[st];
-                L.item0[q - b0 + 1] = L.item0[q - b0] + (int)((chunks + L.cpi - 1) / L.cpi);
-              }
+            p.members.assign(hr.begin() + b0, hr.begin() + std::min(hr.size(), b0 + (size_t)kListMaxRuns));
+            HeadList &L = p.H;
+            L.nruns = (int)p.members.size();
+            L.n = cl.first;
+            L.herm = herm;
+            L.cta0[0] = 0;
+            for (int q = 0; q < L.nruns; ++q) {
+              int ctas = 0;
+              head_plan(p.members[q], &L.apu, &L.splits, &ctas);
+              L.d[q] = reinterpret_cast<const ElRunDesc *>(p.members[q]->desc_dev);
+              L.cta0[q + 1] = L.cta0[q] + ctas;
             }
-            for (size_t q = b0; q < b1; ++q) p.members.push_back(rv[cl.second[q]]);
             prep.push_back(std::move(p));
           }
+        }
+        for (size_t b0 = 0; b0 < cl.second.size(); b0 += kListMaxRuns) {
+          const size_t b1 = std::min(cl.second.size(), b0 + (size_t)kListMaxRuns);
+          Prepared p;
+          p.n = cl.first;
+          p.head = false;
+          p.sm_count = rv[cl.second[b0]]->sm_count;
+          p.stream = cs;
+          for (int st = 0; st < 4; ++st) {
+            ListLaunch &L = p.L[st];
+            L.nruns = (int)(b1 - b0);
+            L.cpi = kListCpiBody;
+            L.item0[0] = 0;
+            for (size_t q = b0; q < b1; ++q) {
+              const heom_run *r = rv[cl.second[q]];
+              const int A = 32 / r->n < 32 ? 32 / r->n : 31;
+              const int64_t chunks = (r->n_ado - r->u_split + A - 1) / A;
+              L.args[q - b0] = group_args_of(r) + st;
+              L.item0[q - b0 + 1] = L.item0[q - b0] + (int)((chunks + L.cpi - 1) / L.cpi);
+            }
+          }
+          for (size_t q = b0; q < b1; ++q) p.members.push_back(rv[cl.second[q]]);
+          prep.push_back(std::move(p));
         }
       }
       rebuilt_at = s;
     }
     for (int st = 0; st < 4 && rc == HEOM_OK; ++st) {
       for (Prepared &p : prep) {
-        if (launch_stage_list(p.kind, p.n, p.L[st], p.stream, p.sm_count)) {
+        if (p.head) {
+          p.H.stage = st;
+          p.H.ch = horner_c(st, h);
+        }
+        if (p.head ? launch_head_list(p.H, p.stream, p.sm_count) : launch_stage_list(p.n, p.L[st], p.stream, p.sm_count)) {
           rc = HEOM_E_CUDA;
           break;
         }
@@ -254,17 +259,17 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       }
       // runs outside the work lists: their own launches, on the caller's stream
       for (int i = 0; i < n_runs && rc == HEOM_OK; ++i) {
-        if (listed[i] || n_steps[i] <= s) continue;
+        if (listed[i] || done[i] || n_steps[i] <= s) continue;
         heom_run *r = rv[i];
         const HornerStage &hs = kHorner[st];
         cudaStream_t own = r->stream;
         r->stream = gs;
-        rc = run_stage(r, view_of(r, hs.zin), view_of(r, hs.y), view_of(r, hs.out), hs.c * h);
+        rc = run_stage(r, view_of(r, hs.zin), view_of(r, hs.y), view_of(r, hs.out), horner_c(st, h));
         r->stream = own;
       }
     }
     for (int i = 0; i < n_runs && rc == HEOM_OK; ++i) {  // step counters and observable records
-      if (n_steps[i] <= s) continue;
+      if (n_steps[i] <= s || done[i]) continue;
       heom_run *r = rv[i];
       ++r->steps_done;
       r->t_fs += h;

@@ -23,17 +23,13 @@ namespace heom {
 static thread_local std::string g_err;
 void set_error(const std::string &msg) { g_err = msg; }
 
-int launch_stage(int precision, const StageCommon &c, double ch, const double *term, const double *H,
-                 const double *Hi, cudaStream_t st, int sm_count) {
+int launch_stage(const StageCommon &c, double ch, const double *term, const double *H, const double *Hi, cudaStream_t st,
+                 int sm_count) {
   if (c.u_end <= c.u_begin) return 0;
-  static int (*const fns[3][4])(const StageCommon &, double, const double *, const double *, const double *,
-                                 cudaStream_t, int) = {
-      {launch_stage_fp64_a, launch_stage_fp64_b, launch_stage_fp64_c, launch_stage_fp64_d},
-      {launch_stage_fp32_a, launch_stage_fp32_b, launch_stage_fp32_c, launch_stage_fp32_d},
-      {launch_stage_head_a, launch_stage_head_b, launch_stage_head_c, launch_stage_head_d}};
+  static int (*const fns[4])(const StageCommon &, double, const double *, const double *, const double *, cudaStream_t,
+                             int) = {launch_stage_fp32_a, launch_stage_fp32_b, launch_stage_fp32_c, launch_stage_fp32_d};
   int rc = 1;
-  if (precision == 0 && c.herm && !c.cplx_h) rc = launch_stage_col(c, ch, term, H, st, sm_count);
-  for (int g = 0; g < 4 && rc == 1; ++g) rc = fns[precision][g](c, ch, term, H, Hi, st, sm_count);
+  for (int g = 0; g < 4 && rc == 1; ++g) rc = fns[g](c, ch, term, H, Hi, st, sm_count);
   if (rc == 1) {
     set_error("stage kernel: n_states not compiled");
     return -1;
@@ -41,10 +37,10 @@ int launch_stage(int precision, const StageCommon &c, double ch, const double *t
   return rc;
 }
 
-int launch_stage_list(int kind, int n, const ListLaunch &L, cudaStream_t st, int sm_count) {
-  int rc = launch_stage_list_a(kind, n, L, st, sm_count);
-  if (rc == 1) rc = launch_stage_list_b(kind, n, L, st, sm_count);
-  if (rc == 1) rc = launch_stage_list_c(kind, n, L, st, sm_count);
+int launch_stage_list(int n, const ListLaunch &L, cudaStream_t st, int sm_count) {
+  int rc = launch_stage_list_a(n, L, st, sm_count);
+  if (rc == 1) rc = launch_stage_list_b(n, L, st, sm_count);
+  if (rc == 1) rc = launch_stage_list_c(n, L, st, sm_count);
   if (rc == 1) set_error("work-list stage kernel: n_states not compiled");
   return rc;
 }
@@ -124,6 +120,8 @@ struct Layout {
   size_t head_bytes, body_bytes;
   size_t total;
 };
+
+constexpr size_t kCountBytes = 128;  // record counter (8 bytes), error flag (8), at 64 the barrier counters
 
 inline size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -389,9 +387,9 @@ Layout make_layout(int n, const Hierarchy &h, int u_split, int precision, int64_
   L.off_gsum = o; o = al(o + (size_t)n_ado * sizeof(double));
   L.off_rec = o; o = al(o + (size_t)std::max<int64_t>(max_records, 1) * (n + 5) * sizeof(double));
   L.off_w = o; o = al(o + (size_t)n * sizeof(double));
-  L.off_cnt = o; o = al(o + 2 * sizeof(int64_t));  // record counter, device error flag
-  // stage arguments of grouped launches: batched column-0 (4 stages x 2 VecRunDesc) or work-list (GroupRunDesc)
-  L.off_desc = o; o = al(o + std::max(8 * sizeof(VecRunDesc), sizeof(GroupRunDesc)));
+  L.off_cnt = o; o = al(o + kCountBytes);  // record counter, device error flag, barrier counters
+  // stage arguments: batched column-0 launches (4 stages x 2 VecRunDesc), or an ElRunDesc and its constants
+  L.off_desc = o; o = al(o + 8 * sizeof(VecRunDesc));
   L.head_bytes = al((size_t)u_split * E * sizeof(double2));
   L.body_bytes = al((size_t)(n_ado - u_split) * *Ep * be);
   for (int c = 0; c < copies; ++c) {
@@ -561,8 +559,6 @@ extern "C" int heom_run_create(const heom_system *sys, const heom_hier *hh, int 
           const double d = v_diag(sys, b, i) - v_diag(sys, b, j);
           r->T[(size_t)i * n + j] += dbath[b] * d * d;
         }
-    r->Ht = r->H;
-    r->Hit = r->Hi;
   }
 
   // ---- rescaling factors s+_l(n), s-_l(n) (section "HEOM formalism", ADO rescaling)
@@ -715,6 +711,7 @@ extern "C" int heom_run_create(const heom_system *sys, const heom_hier *hh, int 
   r->copy_bytes = L.head_bytes + L.body_bytes;
   r->desc_dev = reinterpret_cast<VecRunDesc *>(base + L.off_desc);
   r->err_dev = reinterpret_cast<int *>(base + L.off_cnt + sizeof(int64_t));
+  r->bar_dev = reinterpret_cast<unsigned *>(base + L.off_cnt + 64);
   r->y = view_at(base, L, 0);
   r->zA = view_at(base, L, 1);
   r->zB = view_at(base, L, 2);
@@ -732,7 +729,7 @@ extern "C" int heom_run_create(const heom_system *sys, const heom_hier *hh, int 
     ce = cudaMemcpyAsync(r->recs_body, rbf.data(), rbf.size() * sizeof(rbf[0]), cudaMemcpyHostToDevice, st);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(r->gsum, gs.data(), gs.size() * sizeof(double), cudaMemcpyHostToDevice, st);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(r->w_dev, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (ce == cudaSuccess) ce = cudaMemsetAsync(r->rec_count, 0, 2 * sizeof(int64_t), st);
+  if (ce == cudaSuccess) ce = cudaMemsetAsync(r->rec_count, 0, kCountBytes, st);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(base + L.off_state[0], 0, L.head_bytes + L.body_bytes, st);
   // the host vectors are pageable, so each copy has consumed its source when cudaMemcpyAsync returns
   if (ce != cudaSuccess) { delete r; return cuda_fail("workspace upload", ce); }
@@ -741,6 +738,7 @@ extern "C" int heom_run_create(const heom_system *sys, const heom_hier *hh, int 
   for (int i = 0; i < n * n; ++i) { s0r[i] = sigma0_re[i]; if (sigma0_im) s0i[i] = sigma0_im[i]; }
   *out = r;
   rc = heom_set_ados(r, 0, 1, s0r.data(), s0i.data());
+  if (rc == HEOM_OK && !r->vec) rc = el_upload(r);
   if (rc == HEOM_OK) rc = enqueue_record(r);
   if (rc == HEOM_OK) rc = schedule_new_run(r);
   if (rc != HEOM_OK) { *out = nullptr; delete r; return rc; }
@@ -832,7 +830,7 @@ static int leave_vec(heom_run *r) {
   r->flops_gen = r->flops_full;
   r->flops_herm = r->flops_full;
   reschedule_cached(r);  // the matrix-layout kernels: their own cache entries, else the default
-  return HEOM_OK;
+  return el_upload(r);
 }
 
 extern "C" int heom_set_ados(heom_run *r, int64_t u0, int64_t count, const double *re, const double *im) {
@@ -849,6 +847,7 @@ extern "C" int heom_set_ados(heom_run *r, int64_t u0, int64_t count, const doubl
       if (rc) return rc;
     }
   }
+  const bool was_herm = r->herm;
   if (r->herm && re && im) {  // a non-Hermitian ADO switches the run to the general kernels for good
     const int n = r->n;
     for (int64_t c = 0; c < count && r->herm; ++c) {
@@ -860,6 +859,10 @@ extern "C" int heom_set_ados(heom_run *r, int64_t u0, int64_t count, const doubl
             break;
           }
     }
+  }
+  if (was_herm && !r->herm && r->desc_owner) {  // the element kernels' descriptor says so too
+    const int rc = el_upload(r);
+    if (rc) return rc;
   }
   return io_range(r, r->y, u0, count, const_cast<double *>(re), const_cast<double *>(im), true);
 }
@@ -907,10 +910,8 @@ extern "C" int heom_run_set_field(heom_run *r, const heom_field *f) {
   r->fsig = f->sigma_fs;
   r->fphase = f->phase;
   r->fdet = kCmToRadFs * f->detuning_cm;
-  r->Ht.assign((size_t)n * n, 0.0);
-  r->Hit.assign((size_t)n * n, 0.0);
   r->has_field = true;
-  return HEOM_OK;
+  return el_upload(r);
 }
 
 extern "C" int64_t heom_run_launches(const heom_run *r) { return r ? r->launches : -1; }

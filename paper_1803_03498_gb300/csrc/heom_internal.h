@@ -170,36 +170,13 @@ struct StageArgs {
 #define HEOM_DECLARE_LAUNCH(NAME)                                                                      \
   int NAME(const StageCommon &c, double ch, const double *term, const double *H, const double *Hi, \
            cudaStream_t st, int sm_count);
-HEOM_DECLARE_LAUNCH(launch_stage_fp64_a)
-HEOM_DECLARE_LAUNCH(launch_stage_fp64_b)
-HEOM_DECLARE_LAUNCH(launch_stage_fp64_c)
-HEOM_DECLARE_LAUNCH(launch_stage_fp64_d)
 HEOM_DECLARE_LAUNCH(launch_stage_fp32_a)
 HEOM_DECLARE_LAUNCH(launch_stage_fp32_b)
 HEOM_DECLARE_LAUNCH(launch_stage_fp32_c)
 HEOM_DECLARE_LAUNCH(launch_stage_fp32_d)
-HEOM_DECLARE_LAUNCH(launch_stage_head_a)
-HEOM_DECLARE_LAUNCH(launch_stage_head_b)
-HEOM_DECLARE_LAUNCH(launch_stage_head_c)
-HEOM_DECLARE_LAUNCH(launch_stage_head_d)
 #undef HEOM_DECLARE_LAUNCH
 
-// General stage kernel (gen_kernel.cuh): bath couplings with several states, a time-dependent H and
-// up to kGenMaxStates states.  out1 (c.out) = base1 (c.y) + c1 L zin; out2 = base2 + c2 L zin when
-// out2 is set.  H, Hi, T: host arrays [n][n] (H(t) - h0 and Im H(t) in rad/fs; T_ij the terminator
-// rate of element (i, j)).  kind as launch_stage_vec.
-constexpr int kGenMaxStates = 32;
-template <typename CT>
-struct GenArgs {
-  StageCommon c;
-  StateView base2, out2;
-  CT c1, c2;
-  CT H[kGenMaxStates * kGenMaxStates];
-  CT Hi[kGenMaxStates * kGenMaxStates];
-  CT T[kGenMaxStates * kGenMaxStates];
-};
-int launch_stage_gen(int kind, const StageCommon &c, StateView base2, StateView out2, double c1, double c2,
-                     const double *H, const double *Hi, const double *T, cudaStream_t st, int sm_count);
+constexpr int kGenMaxStates = 32;  // states of general runs (element kernels only)
 
 // Column-form FP64 stage kernel (stage_col.cuh) for Hermitian runs with a real H and 8 <= n <= 16:
 // every lane of a warp owns one column of one part of an ADO's result, so all 32 lanes do FP64 work.
@@ -207,37 +184,88 @@ int launch_stage_gen(int kind, const StageCommon &c, StateView base2, StateView 
 int launch_stage_col(const StageCommon &c, double ch, const double *term, const double *H, cudaStream_t st,
                      int sm_count);
 
-// Work-list launches (stage_list.cuh): one launch covers the same stage of many runs of equal
-// n_states (real H).  A run's stage arguments for such launches live in its workspace.
-template <typename CT>
+// Element kernels (resident.cuh).  Constants of a matrix-layout run, in its workspace, [n][n] row-major
+// and FP64: Re H - h0, Im H, the terminator rate T_ij of element (i, j), the laser field's M+ (NULL: no
+// field), and the terminator Delta_i per state.
+struct ElConsts {
+  const double *H, *Hi, *T, *mup, *term;
+};
+// One stage over [c.u_begin, c.u_end): out = y + c1 L zin, and out2 = y2 + c2 L zin if out2 is set;
+// gr + i gi is the laser field's g(t).
+struct ElStageArgs {
+  StageCommon c;
+  ElConsts k;
+  StateView y2, out2;
+  double c1, c2, gr, gi;
+  int apu, splits;  // ADOs per unit, or (apu = 1) units per ADO (set by the launcher)
+  bool fixed;       // pair kernels: fixed-point commutator (set by the launcher)
+  bool general;     // couplings with several states per bath, a laser field or more than 24 states
+};
+// kind as launch_stage_vec (the FP32 body only for general runs).
+int launch_el_stage(int kind, const ElStageArgs &a, cudaStream_t st, int sm_count);
+
+// One run of an el_run_kernel launch, in the run's workspace.
+struct ElRunDesc {
+  StageCommon c;
+  StateView st[3];  // y, zA, zB
+  ElConsts k;
+  unsigned *bar;    // [2] barrier counters, zero between launches
+  const double *w;
+  double *records;
+  int64_t *rec_count;
+  int64_t max_records;
+  int fp64, pad;
+};
+struct ElEntry {
+  const ElRunDesc *d;
+  int cta0;                  // first CTA of the run
+  int hcta;                  // CTAs of the FP64 part
+  int apu64, split64, apu32;  // units of the FP64 part and of an FP32 body taken by elements
+  int row_bytes;             // shared memory per warp of an FP32 body taken by rows
+  int steps;
+  int stride, first_rec;     // a record every stride steps, the first after first_rec steps (0: none)
+};
+constexpr int kElMaxRuns = 256;  // runs per launch (kernel parameters: about 10 KB)
+struct ElList {
+  ElEntry e[kElMaxRuns];
+  double ch[4];  // the stages' Horner coefficients times h
+  int nruns;
+};
+
+// Work-list launches (stage_list.cuh): one launch covers the same stage of the FP32 bodies of many runs of
+// equal n_states (real H).  A run's stage arguments for such launches live in its workspace.
 struct alignas(16) GroupArgs {
   StageCommon c;
-  CT ch;                           // Horner coefficient times h
-  CT term[kMaxStates];             // terminator Delta per state
-  alignas(16) CT H[kMaxStates * kMaxStates];   // Re H - h0 I, row stride kMaxStates, rad/fs
-};
-// Per run: the four Horner stages of the FP32 body and of the FP64 head (mixed precision).
-struct GroupRunDesc {
-  GroupArgs<float> body[4];
-  GroupArgs<double> head[4];
+  float ch;                           // Horner coefficient times h
+  float term[kMaxStates];             // terminator Delta per state
+  alignas(16) float H[kMaxStates * kMaxStates];   // Re H - h0 I, row stride kMaxStates, rad/fs
 };
 constexpr int kListMaxRuns = 64;  // runs per work-list launch (kernel parameters: about 0.8 KB)
 struct ListLaunch {
-  const void *args[kListMaxRuns];  // GroupArgs of run i for this stage and part (device)
+  const GroupArgs *args[kListMaxRuns];  // arguments of run i for this stage (device)
   int item0[kListMaxRuns + 1];     // run i owns items [item0[i], item0[i + 1]) of cpi chunks each
   int nruns;
   int cpi;
 };
-// One work-list launch of runs of n states: kind 1 = mixed body (FP32), 2 = mixed head (FP64 compute,
-// FP32 body neighbours).  Returns 1 when n is not compiled in the unit.
-int launch_stage_list(int kind, int n, const ListLaunch &L, cudaStream_t st, int sm_count);
-int launch_stage_list_a(int kind, int n, const ListLaunch &L, cudaStream_t st, int sm_count);
-int launch_stage_list_b(int kind, int n, const ListLaunch &L, cudaStream_t st, int sm_count);
-int launch_stage_list_c(int kind, int n, const ListLaunch &L, cudaStream_t st, int sm_count);
+// One work-list launch of runs of n states.  Returns 1 when n is not compiled in the unit.
+int launch_stage_list(int n, const ListLaunch &L, cudaStream_t st, int sm_count);
+int launch_stage_list_a(int n, const ListLaunch &L, cudaStream_t st, int sm_count);
+int launch_stage_list_b(int n, const ListLaunch &L, cudaStream_t st, int sm_count);
+int launch_stage_list_c(int n, const ListLaunch &L, cudaStream_t st, int sm_count);
 
-// precision: 0 = FP64 (compute and storage double), 1 = mixed body (float, float), 2 = mixed head
-// (compute double, body storage float).
-int launch_stage(int precision, const StageCommon &c, double ch, const double *term, const double *H,
+// The FP64 heads of the same runs (resident.cuh): CTAs [cta0[i], cta0[i + 1]) take run i's units of apu ADOs, or (apu = 1)
+// `splits` units of one ADO.
+struct HeadList {
+  const ElRunDesc *d[kListMaxRuns];
+  int cta0[kListMaxRuns + 1];
+  int nruns, n, herm, apu, splits;
+  int stage;   // 0..3
+  double ch;
+};
+int launch_head_list(const HeadList &L, cudaStream_t st, int sm_count);
+
+// The FP32 body of a mixed run on the row kernels (stage_kernel.cuh).
+int launch_stage(const StageCommon &c, double ch, const double *term, const double *H,
                  const double *Hi, cudaStream_t st, int sm_count);
 
 }  // namespace heom

@@ -55,13 +55,14 @@ struct heom_run {
   bool has_field = false;            // laser field set (heom_run_set_field): classic four-copy RK4
   std::vector<double> mup;           // [n][n] M+
   double famp = 0, ftc = 0, fsig = 1, fphase = 0, fdet = 0;  // rad/fs, fs, fs, rad, rad/fs
-  std::vector<double> Ht, Hit;       // H(t) of the current stage (general kernel)
+  double gr = 0, gi = 0;             // the field's g(t) of the current stage
   size_t copy_bytes = 0;             // bytes of one state copy (head + body, matrix layout)
   double bytes_full_y = 0, bytes_full_noy = 0, flops_full = 0;  // matrix-layout accounting
-  heom::VecRunDesc *desc_dev = nullptr;    // [8] stage arguments for batched column-0 launches, or a
-                                           // GroupRunDesc for work-list launches (heom_group_propagate)
-  const void *desc_owner = nullptr;  // the batch whose stage arguments desc_dev holds (or the work-list tag)
-  double desc_dt = 0;                // time step of the work-list stage arguments in desc_dev
+  heom::VecRunDesc *desc_dev = nullptr;    // [8] stage arguments for batched column-0 launches, or the
+                                           // element kernels' ElRunDesc and constants (matrix layout)
+  const void *desc_owner = nullptr;  // the batch whose stage arguments desc_dev holds (or the element kernels' tag)
+  double group_dt = 0;               // time step and herm of the work-list arguments in desc_dev (0: none)
+  bool group_herm = false;
   std::vector<double> term;          // per state
   double max_rate = 0;               // D * max gamma
   // device
@@ -75,6 +76,7 @@ struct heom_run {
   double *records = nullptr;         // [max_records][n + 5]
   double *w_dev = nullptr;           // [n] dipole weights (zeros if none)
   int64_t *rec_count = nullptr;      // device counter of records written
+  unsigned *bar_dev = nullptr;       // [2] barrier counters of el_run_kernel
   int *err_dev = nullptr;            // device flag set by a bounded device-side wait that gave up
   int64_t max_records = 0;
   int64_t records_host = 0;          // records enqueued so far (host view)
@@ -111,11 +113,26 @@ StageCommon common_for(const heom_run *r, StateView zin, StateView y, StateView 
 int launch_head(heom_run *r, StageCommon c, double ch, cudaStream_t s);  // FP64 head launch of a stage
 int launch_body(heom_run *r, StageCommon c, double ch, cudaStream_t s);  // body launch of a stage
 int run_stage(heom_run *r, StateView zin, StateView y, StateView out, double ch);
-void field_H(heom_run *r, double t);  // H(t) of a run with a laser field into r->Ht, r->Hit
+void field_g(heom_run *r, double t);  // g(t) of a run with a laser field into r->gr, r->gi
+
+// Coefficient of stage q of a Horner step of length h.
+inline double horner_c(int q, double h) { return q == 0 ? h / 4 : q == 1 ? h / 3 : q == 2 ? h / 2 : h; }
+
+// the element kernels (resident.cu)
+constexpr double kElMaxCost64 = 1.6e7;  // cycles of one stage on one SM (see el_small)
+constexpr double kElMaxCost32 = 1.5e6;
+ElConsts el_consts_of(const heom_run *r);
+int el_upload(heom_run *r);
+bool el_small(const heom_run *r);
+const GroupArgs *group_args_of(const heom_run *r);
+int el_group_args(heom_run *r, double h, cudaStream_t s);
+void head_plan(const heom_run *r, int *apu, int *splits, int *ctas);
+int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s);
 
 // the launch-schedule autotuner (tuner.cu)
 extern std::atomic<int> g_autotune;  // timed launches per candidate at creation (0: off)
 int ilog2(int64_t x);
+bool capturing(cudaStream_t s);  // s is being captured into a graph (or cannot be asked)
 std::vector<heom_schedule> candidates(int layout);
 bool cache_get(const std::array<int, 7> &k, heom_schedule *out);
 void cache_put(const std::array<int, 7> &k, const heom_schedule &s);

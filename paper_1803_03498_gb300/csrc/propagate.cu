@@ -82,15 +82,29 @@ static int join_head(heom_run *r, cudaStream_t hs) {
   return e == cudaSuccess ? HEOM_OK : cuda_fail("head stream join", e);
 }
 
+// Arguments of a one-output stage on the element kernels.
+static ElStageArgs el_args(const heom_run *r, const StageCommon &c, double ch) {
+  ElStageArgs a{};
+  a.c = c;
+  a.k = el_consts_of(r);
+  a.y2 = a.out2 = StateView{nullptr, nullptr};
+  a.c1 = ch;
+  a.general = r->gen;
+  if (r->has_field) {
+    a.gr = r->gr;
+    a.gi = r->gi;
+  }
+  return a;
+}
+
 // The FP64 head launch (ADOs u < u_split) of a mixed-precision stage, on stream s.
 int heom::launch_head(heom_run *r, StageCommon c, double ch, cudaStream_t s) {
   c.u_begin = 0;
   c.u_end = r->u_split;
   c.occ_pct = r->sched[1].occupancy_pct;
   c.cpw = r->sched[1].chunks_per_warp;
-  const double *Hi = r->cplx_h ? r->Hi.data() : nullptr;
   const int rc = r->vec ? launch_stage_vec(2, c, ch, r->term.data(), r->H.data(), s, r->sm_count)
-                        : launch_stage(2, c, ch, r->term.data(), r->H.data(), Hi, s, r->sm_count);
+                        : launch_el_stage(2, el_args(r, c, ch), s, r->sm_count);
   if (rc) return HEOM_E_CUDA;
   ++r->launches;
   return HEOM_OK;
@@ -109,61 +123,58 @@ int heom::launch_body(heom_run *r, StageCommon c, double ch, cudaStream_t s) {
   if (r->vec) {
     rc = launch_stage_vec(fp64 ? 0 : 1, c, ch, r->term.data(), r->H.data(), s, r->sm_count);
   } else if (fp64) {
-    rc = launch_stage(0, c, ch, r->term.data(), r->H.data(), Hi, s, r->sm_count);
+    if (el_small(r) || !r->herm || r->cplx_h) rc = 1;
+    else rc = launch_stage_col(c, ch, r->term.data(), r->H.data(), s, r->sm_count);
+    if (rc == 1) rc = launch_el_stage(0, el_args(r, c, ch), s, r->sm_count);
   } else {
     if (r->precision == HEOM_SPLIT_TF32 && r->herm && !r->cplx_h) {  // tensor-core commutator
       rc = launch_stage_tc_a(c, ch, r->term.data(), r->H.data(), s, r->sm_count);
       if (rc == 1) rc = launch_stage_tc_b(c, ch, r->term.data(), r->H.data(), s, r->sm_count);
     }
-    if (rc == 1) rc = launch_stage(1, c, ch, r->term.data(), r->H.data(), Hi, s, r->sm_count);
+    if (rc == 1) rc = launch_stage(c, ch, r->term.data(), r->H.data(), Hi, s, r->sm_count);
   }
   if (rc) return HEOM_E_CUDA;
   ++r->launches;
   return HEOM_OK;
 }
 
-// H(t) of a run with a laser field (Eq. h-field-rwa in the rotating frame):
-// H - g M+ - conj(g) (M+)^T, g = amp exp(-(t - t_c)^2 / (2 sigma^2)) exp(-i (Delta t + phi)).
-void heom::field_H(heom_run *r, double t) {
-  const int n = r->n;
+// g(t) of a run with a laser field (Eq. h-field-rwa in the rotating frame), from which the kernels form
+// H(t) = H - g M+ - conj(g) (M+)^T:  g = amp exp(-(t - t_c)^2 / (2 sigma^2)) exp(-i (Delta t + phi)).
+void heom::field_g(heom_run *r, double t) {
   const double x = (t - r->ftc) / r->fsig;
   const double env = r->famp * std::exp(-0.5 * x * x);
   const double ph = r->fdet * t + r->fphase;
-  const double gr = env * std::cos(ph), gi = -env * std::sin(ph);
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) {
-      const double a = r->mup[(size_t)i * n + j], b = r->mup[(size_t)j * n + i];
-      r->Ht[(size_t)i * n + j] = r->H[(size_t)i * n + j] - gr * (a + b);
-      r->Hit[(size_t)i * n + j] = r->Hi[(size_t)i * n + j] - gi * a + gi * b;
-    }
+  r->gr = env * std::cos(ph);
+  r->gi = -env * std::sin(ph);
 }
 
-// One stage on the general kernel: out1 = base1 + c1 L zin and, if out2 is set, out2 = base2 + c2 L zin,
-// with H(t) from r->Ht (field) or the constant H.
+// One stage of a general run: out1 = base1 + c1 L zin and, if out2 is set, out2 = base2 + c2 L zin, with H(t)
+// from r->gr, r->gi (field) or the constant H.
 static int run_stage_gen(heom_run *r, StateView zin, StateView b1, StateView o1, double c1, StateView b2, StateView o2,
                          double c2) {
-  StageCommon c = common_for(r, zin, b1, o1);
-  const double *H = r->has_field ? r->Ht.data() : r->H.data();
-  const double *Hi = r->has_field ? r->Hit.data() : r->Hi.data();
+  const StageCommon c = common_for(r, zin, b1, o1);
+  ElStageArgs a = el_args(r, c, c1);
+  a.y2 = b2;
+  a.out2 = o2;
+  a.c2 = c2;
   const bool fp64 = r->precision == HEOM_FP64;
   cudaStream_t hs = r->stream;
   int rc;
   if (!fp64) {  // FP64 head (levels 0, 1) on the side stream
     hs = fork_head(r);
-    StageCommon ch = c;
-    ch.u_begin = 0;
-    ch.u_end = r->u_split;
-    ch.occ_pct = r->sched[1].occupancy_pct;
-    if (launch_stage_gen(2, ch, b2, o2, c1, c2, H, Hi, r->T.data(), hs, r->sm_count)) return HEOM_E_CUDA;
+    ElStageArgs ah = a;
+    ah.c.u_begin = 0;
+    ah.c.u_end = r->u_split;
+    ah.c.occ_pct = r->sched[1].occupancy_pct;
+    if (launch_el_stage(2, ah, hs, r->sm_count)) return HEOM_E_CUDA;
     ++r->launches;
   }
-  c.u_begin = fp64 ? 0 : r->u_split;
-  c.u_end = (int)r->n_ado;
-  c.occ_pct = r->sched[0].occupancy_pct;
-  if (c.u_end > c.u_begin) {
+  a.c.u_begin = fp64 ? 0 : r->u_split;
+  a.c.u_end = (int)r->n_ado;
+  a.c.occ_pct = r->sched[0].occupancy_pct;
+  if (a.c.u_end > a.c.u_begin) {
     if ((rc = timed_begin(r))) return rc;
-    if (launch_stage_gen(fp64 ? 0 : 1, c, b2, o2, c1, c2, H, Hi, r->T.data(), r->stream, r->sm_count))
-      return HEOM_E_CUDA;
+    if (launch_el_stage(fp64 ? 0 : 1, a, r->stream, r->sm_count)) return HEOM_E_CUDA;
     ++r->launches;
     if ((rc = timed_end(r, r->bytes_stage_y))) return rc;
   }
@@ -246,12 +257,12 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
     for (int64_t s = 0; s < n_steps; ++s) {
       const double t = t0 + (double)s * h;
       int rc;
-      field_H(r, t);
+      field_g(r, t);
       if ((rc = run_stage_gen(r, r->y, r->y, r->zA, h / 2, r->y, r->zC, h / 6))) return rc;
-      field_H(r, t + h / 2);
+      field_g(r, t + h / 2);
       if ((rc = run_stage_gen(r, r->zA, r->y, r->zB, h / 2, r->zC, r->zC, h / 3))) return rc;
       if ((rc = run_stage_gen(r, r->zB, r->y, r->zA, h, r->zC, r->zC, h / 3))) return rc;
-      field_H(r, t + h);
+      field_g(r, t + h);
       if ((rc = run_stage_gen(r, r->zA, r->zC, r->y, h / 6, none, none, 0.0))) return rc;
       ++r->steps_done;
       r->t_fs = t0 + (double)(s + 1) * h;
@@ -260,6 +271,8 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
     }
     return HEOM_OK;
   }
+  if (n_steps > 0 && el_small(r) && !r->timing && !capturing(r->stream))
+    return el_propagate(&r, 1, h, &n_steps, obs_stride, r->stream);
   for (int64_t s = 0; s < n_steps; ++s) {
     int rc;
     if ((rc = run_stage(r, r->y, r->y, r->zA, h / 4))) return rc;
@@ -312,7 +325,7 @@ extern "C" int heom_observables(heom_run *r, double *out, int64_t cap_records, i
 extern "C" int heom_rhs_eval(heom_run *r, int64_t u0, int64_t count, double *re, double *im) {
   if (!r) { set_error("heom_rhs_eval: NULL run"); return HEOM_E_ARG; }
   StateView none{nullptr, nullptr};
-  if (r->has_field) field_H(r, r->t_fs);  // L at the current time
+  if (r->has_field) field_g(r, r->t_fs);  // L at the current time
   int rc = run_stage(r, r->y, none, r->zA, 1.0);
   if (rc) return rc;
   cudaError_t e = cudaStreamSynchronize(r->stream);

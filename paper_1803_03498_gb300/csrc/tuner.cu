@@ -73,7 +73,7 @@ void cache_put(const std::array<int, 7> &k, const heom_schedule &s) {
   g_tune_cache[k] = s;
 }
 
-static bool capturing(cudaStream_t s) {
+bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
 }
