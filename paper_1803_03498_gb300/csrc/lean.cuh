@@ -162,7 +162,7 @@ __device__ __forceinline__ double2 lean_comm(const LeanSmem &s, const LeanPair &
     cr = ar - br;
     ci = ai - bi;
   } else if (fx_ok(hk, kx) && fx_ok(hk, ky)) {
-    FxSum r{0, 0, 0}, m{0, 0, 0};
+    FxSum r, m;
     const int4 *zi = s.tile + (p.la * n + p.i) * n, *zj = s.tile + p.la * n * n + p.j;
     const int2 *hi_ = s.H + p.i * n, *hj = s.H + p.j;
 #pragma unroll 2

@@ -21,27 +21,18 @@
 //    of its own that keep their ADOs, constants and link ranges in shared memory; a barrier of the
 //    run's CTAs (a counter in the run's workspace) follows every stage.  A stage then costs one barrier
 //    and one round trip to L2 instead of a kernel launch or two.
-// Arithmetic forms (FORM): kElFixed -- FP64 runs and heads, the commutator in fixed point (below);
+// Arithmetic forms (FORM): kElFixed -- FP64 runs and heads, the commutator in fixed point (fixed_point.cuh);
 // kElGeneral -- FP32 runs of the general kind; kElRowOrder -- FP32 non-Hermitian runs in el_run_kernel, every
 // sum in the order of stage_kernel's shared-memory path, so that the results equal that kernel's bit for
 // bit (FP32 Hermitian bodies there run the row kernel's own code, row_body).
 //
-// Fixed-point commutator.  GB300 issues one FP64 FMA per 64 clocks and SM partition (measured: 18.7 clocks
-// per warp instruction and SM), but two 32 x 32 + 64 bit integer multiply-adds per clock and SM (measured
-// 1.92), so a product sum in exact integers costs a ninth of the FP64 one.  H and the real and the imaginary
-// part of a tile are scaled by a power of two each (the largest element's) and rounded to 2 LB bits, kept as two
-// signed limbs of LB bits; sums of limb products are exact in 64 bits (LB = 29 for up to 32 terms, 28 for up
-// to 128), and the total, again below 2^62, is rounded once to FP64.  The idea is the splitting of Ozaki, Ogita,
-// Oishi and Rump (Numer. Algorithms 59, 2012), with integers in place of short floating-point slices.
-// The rounding of an element is at most 2^-(2 LB) of the largest one, below FP64's own half ulp of that element, and
-// no sum rounds on the way: against 64-bit sums in higher precision the error is smaller than that of the
-// FP64 FMA chain.  A tile with Inf, NaN or exponents near the ends of the range takes the FMA chain.
 #pragma once
 #include <cuda_runtime.h>
 
 #include <cstdint>
 #include <type_traits>
 
+#include "fixed_point.cuh"
 #include "heom_internal.h"
 #include "record.cuh"
 #include "stage_kernel.cuh"
@@ -155,59 +146,6 @@ __device__ __forceinline__ ElSmem<CT> el_carve(unsigned char *p, int n, int cnt,
 
 __host__ __device__ inline int el_pairs(int n, int herm) { return herm ? n * (n + 1) / 2 : n * n; }
 
-// ---- fixed point -----------------------------------------------------------------------------------
-
-// |x| as an ordered integer (0 only for zero): the high word, its last bit set if only the low word is not zero.
-__device__ __forceinline__ int fx_key(double x) {
-  const int h = __double2hiint(x) & 0x7fffffff;
-  return h | (h == 0 && __double2loint(x) != 0);
-}
-__device__ __forceinline__ int fx_exp(int key) { return max(key >> 20, 1); }
-
-// x as limbs of lb bits, x = (hi 2^lb + lo) 2^(e - 1022 - (2 lb - 1)), for |x| < 2^(e - 1022): round to nearest.
-__device__ __forceinline__ int2 fx_split(double x, int e, int lb) {
-  const int h = __double2hiint(x);
-  int ex = (h >> 20) & 0x7ff;
-  unsigned long long m = ((unsigned long long)(unsigned)(h & 0xfffff) << 32) | (unsigned)__double2loint(x);
-  if (ex != 0) m |= 1ull << 52;
-  else ex = 1;
-  const int s = ex - e + 2 * lb - 54;
-  unsigned long long u = s >= 0 ? m << s : s > -60 ? (m + (1ull << (-s - 1))) >> -s : 0ull;
-  const long long v = h < 0 ? -(long long)u : (long long)u;
-  const int lo = (int)((unsigned)v << (32 - lb)) >> (32 - lb);
-  return make_int2((int)((v - lo) >> lb), lo);
-}
-
-// k 2^p rounded to nearest even; the caller keeps the result in FP64's normal range.
-__device__ __forceinline__ double fx_double(long long k, int p) {
-  unsigned long long u = k < 0 ? 0ull - (unsigned long long)k : (unsigned long long)k;
-  const int lz = __clzll((long long)u);
-  u <<= (lz & 63);
-  unsigned long long m = u >> 11;
-  const unsigned r = (unsigned)u & 0x7ff;
-  m += (r + ((unsigned)m & 1)) > 0x400;
-  unsigned long long b = ((unsigned long long)(1085 - lz + p) << 52) + m;
-  b = u ? b | (k < 0 ? 1ull << 63 : 0ull) : 0ull;
-  return __longlong_as_double((long long)b);
-}
-
-// a product sum in three parts: hi hi, cross, lo lo
-struct FxSum {
-  long long hh, x, ll;
-  __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
-    hh += (long long)ah * bh;
-    x += (long long)ah * bl;
-    x += (long long)al * bh;
-    ll += (long long)al * bl;
-  }
-  __device__ __forceinline__ long long total(int lb) const {  // in units of hi hi, rounded
-    return hh + ((x + (ll >> lb) + (1ll << (lb - 1))) >> lb);
-  }
-};
-
-// Limb bits: sums of 2 n (real H) or 4 n products stay below 2^63.
-__device__ __forceinline__ int fx_bits(int n, bool cplx) { return !cplx && n <= 16 ? 29 : 28; }
-
 // Constants and the pair table into shared memory (followed by a __syncthreads of the caller).
 // gr, gi: the laser field's g(t) (0 without a field): H(t) = H - g M+ - conj(g) (M+)^T.
 template <typename CT>
@@ -298,7 +236,7 @@ template <bool CPLX>
 __device__ __forceinline__ void el_fix_comm(const ElSmem<double> &s, int n, int la, int pitch, int i, int j, double &cr,
                                             double &ci) {
   const int lb = fx_bits(n, CPLX);
-  FxSum r{0, 0, 0}, m{0, 0, 0};
+  FxSum r, m;
   const int4 *z = reinterpret_cast<const int4 *>(s.tile) + la * pitch;
   const int4 *zi = z + i * n, *zj = z + j;
   const int2 *hi_ = reinterpret_cast<const int2 *>(s.H) + i * n, *hj = reinterpret_cast<const int2 *>(s.H) + j;
@@ -323,12 +261,6 @@ __device__ __forceinline__ void el_fix_comm(const ElSmem<double> &s, int n, int 
   const int eh = fx_exp(*s.hkey) - 2042 - 2 * lb;
   cr = fx_double(r.total(lb), eh + fx_exp(s.key[2 * la]));
   ci = fx_double(m.total(lb), eh + fx_exp(s.key[2 * la + 1]));
-}
-
-// Whether the fixed-point commutator of a tile with this key stays in FP64's normal range (or is exactly zero).
-__device__ __forceinline__ bool fx_ok(int hkey, int key) {
-  const int e = (hkey >> 20) + (key >> 20);
-  return hkey < 0x7ff00000 && key < 0x7ff00000 && (hkey == 0 || key == 0 || (e >= 1120 && e <= 3000));
 }
 
 // The same by FP64 FMAs, from global memory.

@@ -11,28 +11,35 @@
 // a column part, and a link adds R v_sj to row s, conj(R) v_is = conj(R v_si) to column s and
 // 2 Re(R) v_ss to the diagonal (see LinkRec).
 //
-// GB300's FP64 pipe retires 2 FMAs per clock per SM, so this kernel is bound by its FP64 instruction
-// count, and a warp instruction costs the same whether 28 or 32 lanes do useful work.  The row form
-// of stage_kernel maps lane (a, i) to row i of ADO a: at N = 14 two ADOs fill 28 of 32 lanes.  Here a
-// lane owns one column of one part: lane (a, p, j) computes column j of Q_re (p = 0, from H Im s) or
-// of Q_im (p = 1, from -H Re s) of ADO a -- 2N columns per ADO.  A warp takes chunks of G consecutive
-// ADOs, G chosen so that 2 N G is a multiple of 32, and covers their 2 N G columns in P = 2 N G / 32
+// Bound and form: GB300 issues one FP64 instruction per 64 clocks and SM partition (18.7 clocks per SM measured), two
+// 32 x 32 + 64 bit integer multiply-adds per clock and SM.  The commutator, 2 N^3 multiply-adds per ADO, therefore runs
+// in exact integers (fixed_point.cuh: two limbs of 29 bits, one rounding at the end of a sum), and the FP64 pipe keeps
+// what is cheaper there than in integers: the sums' conversion (2 additions), the decay, the links (2 per
+// record and lane), R and the RK4 combination (4 per pair of elements).  A lane owns one column of one part: lane (a, p, j)
+// computes column j of Q_re (p = 0, from H Im s) or of Q_im (p = 1, from -H Re s) of ADO a -- 2N columns
+// per ADO -- so the scale of its operands is its own column's largest element, without a word to other lanes, and
+// the limbs of H enter every multiply-add as kernel-parameter (constant-bank) operands.  A warp takes chunks of G
+// consecutive ADOs, G chosen so that 2 N G is a multiple of 32, and covers their 2 N G columns in P = 2 N G / 32
 // passes with every lane busy (N = 14: 8 ADOs in 7 passes).  Per pass a lane
 //   - loads column j of its ADO's zin tile from global memory (the 2N lanes of an ADO read whole rows:
-//     coalesced), H enters every FMA as a kernel-parameter (constant-bank) operand;
-//   - accumulates the N entries of its column of H (Im s) or -H (Re s) and adds coef * (own part);
-//   - writes the column into its ADO's slot of a per-warp ring of Q tiles in shared memory.
-// An ADO whose last column was computed in this pass is finalised by lanes (p, j) of the warp: the
+//     coalesced) and splits the part it multiplies into limbs;
+//   - forms the N entries of its column of H (Im s) or -H (Re s), each a sum of 4 N integer products, plus
+//     coef * (own part);
+//   - writes the column in FP64 into its ADO's slot of a per-warp ring of Q tiles in shared memory.
+// An ADO whose last column was computed in this pass is finalised by the warp: the
 // row s of every linked neighbour (gathered into shared memory by cp.async while the pass computed)
-// is added to row s of Q, records in order; then R_ij = Q_ij + conj(Q_ji) and out = y + ch R leave
-// with coalesced loads and stores.  Warps are independent (only __syncwarp).  Every output element
-// sums the same terms in the same order under every launch schedule.
+// is added to row s of Q, records in order; then the lanes take the pairs i <= j: R_ij = Q_ij + conj(Q_ji),
+// out = y + ch R, written to (i, j) and, conjugated, to (j, i).  Warps are independent (only __syncwarp).  Every output
+// element sums the same terms in the same order under every launch schedule.
+// A column with Inf, NaN or exponents near the ends of the range takes FP64 FMAs instead.
 #pragma once
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
+#include "fixed_point.cuh"
 #include "heom_internal.h"
 
 namespace heom {
@@ -134,8 +141,33 @@ __device__ __forceinline__ void col_links(const LinkRec<double> *rec, int nr, co
   if (cur >= 0) qp[cur * N + j] = acc;
 }
 
+constexpr int kColBits = 29;  // sums of N <= 16 products of 2^56 and twice as many cross products fit 63 bits
+
+struct ColArgs {
+  StageCommon c;
+  double ch;
+  int ex;                                // |H| < 2^(ex - 1022)
+  double term[kMaxStates];               // terminator Delta per state
+  double H[kMaxStates * kMaxStates];     // Re H - h0 I, rad/fs (columns out of range)
+  int2 Hx[kMaxStates * kMaxStates];      // its limbs
+};
+
+// Column j of part p of -i H s + coef s by FP64 FMAs, into q[i * N + j].
 template <int N>
-__global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(const __grid_constant__ StageArgs<double> a) {
+__device__ __noinline__ void col_fma(const ColArgs &a, const double2 *zt, int p, int j, double g, double *q) {
+  for (int i = 0; i < N; ++i) {
+    double acc = 0;
+    for (int k = 0; k < N; ++k) {
+      const double2 z = zt[k * N];
+      acc = fma(a.H[i * kMaxStates + k], p ? -z.x : z.y, acc);
+    }
+    const double2 z = zt[i * N];
+    q[i * N + j] = fma(i == j ? -0.5 * g : fma(-0.5, g, -a.term[i]), p ? z.y : z.x, acc);
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(const __grid_constant__ ColArgs a) {
   using S = ColShape<N>;
   using W = ColSmem<N>;
   constexpr int C = S::C, G = S::G, P = S::P, E = S::E, RB = S::RB;
@@ -201,27 +233,34 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
         col_gather<N>(c, zin, Ep, recb + k * RB, k == 0 ? nrf0 : nrf1, gbuf + k * RB * N, lane);
       if (act) {
         // p = 0: Q_re = H Im s + coef Re s;  p = 1: Q_im = -H Re s + coef Im s
-        double src[N], own[N];
+        int key = 0;
 #pragma unroll
-        for (int k = 0; k < N; ++k) {
-          src[k] = p ? col_neg(zc[k].x) : zc[k].y;
-          own[k] = p ? zc[k].y : zc[k].x;
-        }
-        double acc[N];
-#pragma unroll
-        for (int i = 0; i < N; ++i) acc[i] = 0.0;
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-#pragma unroll
-          for (int i = 0; i < N; ++i) acc[i] = fma(a.H[i * kMaxStates + k], src[k], acc[i]);
-        }
+        for (int k = 0; k < N; ++k) key = max(key, fx_key(p ? zc[k].x : zc[k].y));
         double *qs = qring + (ad % S::RING) * 2 * E + p * E;
-        const double *cf = coef + ad * N;
-        const double gd = gh[ad];
+        if (fx_ok(a.ex << 20, key)) {
+          const int ex = fx_exp(key);
+          int2 src[N];
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-          const double ci = (i == j) ? gd : cf[i];
-          qs[i * N + j] = fma(ci, own[i], acc[i]);
+          for (int k = 0; k < N; ++k) src[k] = fx_split(p ? col_neg(zc[k].x) : zc[k].y, ex, kColBits);
+          const double *cf = coef + ad * N;
+          const double gd = gh[ad];
+          const int e2 = key ? a.ex - 2042 - 2 * kColBits + ex : 0;  // a zero column: any scale in range
+          const double *zo = reinterpret_cast<const double *>(zin + (int64_t)(u0 + ad) * Ep + j) + p;  // own part
+          // rows in a loop: unrolled over them (2700 instructions) the code outgrew the instruction cache and the kernel
+          // took 20 ms at the LHCII size
+#pragma unroll 2
+          for (int i = 0; i < N; ++i) {
+            const double own = zo[2 * i * N], ci = i == j ? gd : cf[i];
+            FxSum r;
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+              const int2 hx = a.Hx[i * kMaxStates + k];
+              r.add(hx.x, hx.y, src[k].x, src[k].y);
+            }
+            qs[i * N + j] = fma(ci, own, fx_double_add(r.total(kColBits), e2));
+          }
+        } else {
+          col_fma<N>(a, zin + (int64_t)(u0 + ad) * Ep + j, p, j, c.gsum[u0 + ad], qs);
         }
       }
       col_wait_all();  // gathers
@@ -245,20 +284,29 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
           col_links<N>(recb + k * RB, nr, gbuf + k * RB * N, qs, lane);
         }
         __syncwarp();
-        if (lane < C) {  // R = Q + Q^dagger, out = y + ch R; lane (pp, jj) writes part pp of column jj
-          const int pp = lane / N, jj = lane - pp * N;
-          const double *qp = qs + pp * E;
-          const int64_t base = 2 * ((int64_t)u * Ep + jj) + pp;  // element (i, jj), part pp: + 2 N i
-          double yr[N];
-          if (has_y) {
+        {  // R = Q + Q^dagger, out = y + ch R: lane t takes pairs t, t + 32, ... (i <= j, row by row)
+          const double2 *y2 = reinterpret_cast<const double2 *>(yv) + (int64_t)u * Ep;
+          double2 *o2 = reinterpret_cast<double2 *>(out) + (int64_t)u * Ep;
+          constexpr int PR = N * (N + 1) / 2;
 #pragma unroll
-            for (int i = 0; i < N; ++i) yr[i] = yv[base + 2 * N * i];
-          }
-          const double sg = pp ? -1.0 : 1.0;  // Re R symmetric, Im R antisymmetric
+          for (int t0 = 0; t0 < PR; t0 += 32) {
+            const int t = t0 + lane;
+            if (t < PR) {
+              // row of pair t: the largest i with i N - i (i - 1) / 2 <= t
+              int i = 0;
 #pragma unroll
-          for (int i = 0; i < N; ++i) {
-            const double r = fma(sg, qp[jj * N + i], qp[i * N + jj]);
-            out[base + 2 * N * i] = has_y ? fma(ch, r, yr[i]) : ch * r;
+              for (int w = 1; w < N; ++w) i += t >= w * N - w * (w - 1) / 2;
+              const int jj = t - (i * N - i * (i - 1) / 2) + i;
+              double2 yr = make_double2(0, 0);
+              if (has_y) yr = y2[i * N + jj];
+              const double rx = qs[i * N + jj] + qs[jj * N + i];  // Re R symmetric, Im R antisymmetric
+              const double ry = qs[E + i * N + jj] - qs[E + jj * N + i];
+              double2 o;
+              o.x = has_y ? fma(ch, rx, yr.x) : ch * rx;
+              o.y = has_y ? fma(ch, ry, yr.y) : ch * ry;
+              o2[i * N + jj] = o;
+              if (i != jj) o2[jj * N + i] = make_double2(o.x, col_neg(o.y));
+            }
           }
         }
         __syncwarp();
@@ -269,17 +317,29 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
 }
 
 template <int N>
-int launch_col(const StageCommon &c, double ch, const double *term, const double *H, cudaStream_t st, int sm_count) {
-  StageArgs<double> a;
+int launch_col(const StageCommon &c, double ch, const double *term, const double *H, cudaStream_t st,
+               int sm_count) {
+  ColArgs a;
   a.c = c;
   a.ch = ch;
+  double top = 0;
+  for (int i = 0; i < c.n * c.n; ++i) top = std::max(top, std::fabs(H[i]));
+  a.ex = top > 0 && std::isfinite(top) ? std::min(std::max(std::ilogb(top) + 1023, 1), 2046) : top > 0 ? 2047 : 1023;
   for (int i = 0; i < kMaxStates; ++i) a.term[i] = (i < c.n) ? term[i] : 0.0;
   for (int i = 0; i < kMaxStates * kMaxStates; ++i) {
     a.H[i] = 0.0;
-    a.Hi[i] = 0.0;
+    a.Hx[i] = make_int2(0, 0);
   }
   for (int i = 0; i < c.n; ++i)
-    for (int j = 0; j < c.n; ++j) a.H[i * kMaxStates + j] = H[i * c.n + j];
+    for (int j = 0; j < c.n; ++j) {
+      const double h = H[i * c.n + j];
+      a.H[i * kMaxStates + j] = h;
+      if (a.ex == 2047) continue;
+      // as fx_split: |h| < 2^(ex - 1022), rounded to 2 kColBits - 1 bits
+      const long long v = std::llrint(std::ldexp(h, 2 * kColBits - 1 - (a.ex - 1022)));
+      const long long lo = ((v + (1ll << (kColBits - 1))) & ((1ll << kColBits) - 1)) - (1ll << (kColBits - 1));
+      a.Hx[i * kMaxStates + j] = make_int2((int)((v - lo) >> kColBits), (int)lo);
+    }
   constexpr int WARPS = ColShape<N>::WARPS;
   const size_t smem = (size_t)WARPS * ColSmem<N>::total;
   static int per_sm = 0;
