@@ -124,6 +124,8 @@ constexpr double kElMaxCost32 = 1.5e6;
 ElConsts el_consts_of(const heom_run *r);
 int el_upload(heom_run *r);
 bool el_small(const heom_run *r);
+bool col_small(const heom_run *r);  // column-0 runs (column_run.cuh)
+int col_propagate(heom_run *r, double h, int64_t steps, int64_t stride, cudaStream_t s);
 const GroupArgs *group_args_of(const heom_run *r);
 int el_group_args(heom_run *r, double h, cudaStream_t s);
 void head_plan(const heom_run *r, int *apu, int *splits, int *ctas);

@@ -273,6 +273,7 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
   }
   if (n_steps > 0 && el_small(r) && !r->timing && !capturing(r->stream))
     return el_propagate(&r, 1, h, &n_steps, obs_stride, r->stream);
+  if (n_steps > 0 && col_small(r) && !r->timing && !capturing(r->stream)) return col_propagate(r, h, n_steps, obs_stride, r->stream);
   for (int64_t s = 0; s < n_steps; ++s) {
     int rc;
     if ((rc = run_stage(r, r->y, r->y, r->zA, h / 4))) return rc;

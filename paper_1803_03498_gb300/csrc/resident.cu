@@ -9,6 +9,7 @@
 #include "heom_internal.h"
 #include "heom_run.h"
 #include "resident.cuh"
+#include "column_run.cuh"
 
 namespace heom {
 
@@ -440,6 +441,76 @@ int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *ste
     if (rs[kind].empty()) continue;
     const int rc = fns[kind](rs[kind].data(), (int)rs[kind].size(), h, st[kind].data(), stride, s);
     if (rc != HEOM_OK) return rc;
+  }
+  return HEOM_OK;
+}
+
+// ---- column-0 runs --------------------------------------------------------------------------------------
+
+// CTAs and ADOs per CTA of a part of `ados` ADOs: an element per thread.
+static void col_part(int n, int64_t ados, int *ctas, int *apu) {
+  *apu = std::max(1, kColThreads / n);
+  *ctas = (int)((ados + *apu - 1) / *apu);
+}
+
+// Column-0 runs whose elements have a thread each on the GPU (two CTAs of 256 per SM): up to 77,824 elements, e.g. 9,700
+// ADOs of 8 states.  FP64 parts are held to four warps per SM, where their pipe is no bound yet.
+bool col_small(const heom_run *r) {
+  if (!r->vec) return false;
+  const int64_t n64 = r->precision == HEOM_FP64 ? r->n_ado : r->u_split;
+  int c64, c32, apu;
+  col_part(r->n, n64, &c64, &apu);
+  col_part(r->n, r->n_ado - n64, &c32, &apu);
+  return (int64_t)c64 + c32 <= 2 * (int64_t)r->sm_count && n64 * r->n <= 128 * (int64_t)r->sm_count;
+}
+
+int col_propagate(heom_run *r, double h, int64_t steps, int64_t stride, cudaStream_t s) {
+  ColRunArgs a{};
+  const StateView none{nullptr, nullptr};
+  ElRunDesc &d = a.d;
+  d.c = common_for(r, none, none, none);
+  d.st[0] = r->y;
+  d.st[1] = r->zA;
+  d.st[2] = r->zB;
+  d.bar = r->bar_dev;
+  d.w = r->w_dev;
+  d.records = r->records;
+  d.rec_count = r->rec_count;
+  d.max_records = r->max_records;
+  d.fp64 = r->precision == HEOM_FP64;
+  for (int q = 0; q < 4; ++q) a.ch[q] = horner_c(q, h);
+  for (int i = 0; i < r->n; ++i) {
+    a.term[i] = r->term[i];
+    for (int j = 0; j < r->n; ++j) a.H[i * kMaxStates + j] = r->H[(size_t)i * r->n + j];
+  }
+  const int64_t n64 = d.fp64 ? r->n_ado : r->u_split;
+  int c32;
+  col_part(r->n, n64, &a.hcta, &a.apu64);
+  col_part(r->n, r->n_ado - n64, &c32, &a.apu32);
+  // a short FP64 part spreads further: its warps wait for their SM partition's pipe
+  if (!d.fp64) {
+    const int spread = std::max(1, 2 * r->sm_count - c32), per = std::max<int>(1, (int)((n64 + spread - 1) / spread));
+    a.apu64 = std::min(a.apu64, std::max(per, std::max(1, 128 / r->n)));
+    a.hcta = (int)((n64 + a.apu64 - 1) / a.apu64);
+  }
+  const size_t smem = std::max(col_smem_bytes(r->n, a.apu64, 8), col_smem_bytes(r->n, a.apu32, 4));  // below 48 KB
+  for (int64_t at = 0; at < steps;) {
+    a.steps = (int)std::min<int64_t>(kElSteps * 2, steps - at);  // about a millisecond
+    a.stride = (int)std::min<int64_t>(stride, 1 << 30);
+    a.first_rec = 0;
+    if (stride > 0) {
+      const int64_t first = stride - r->steps_done % stride;
+      a.first_rec = first <= a.steps ? (int)first : 0;
+    }
+    void *args[] = {&a};
+    cudaError_t e = cudaLaunchCooperativeKernel((const void *)col_run_kernel, dim3(a.hcta + c32), dim3(kColThreads), args, smem, s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail("column run kernel launch", e);
+    if (stride > 0) r->records_host += (r->steps_done + a.steps) / stride - r->steps_done / stride;
+    r->steps_done += a.steps;
+    for (int x = 0; x < a.steps; ++x) r->t_fs += h;
+    ++r->launches;
+    at += a.steps;
   }
   return HEOM_OK;
 }

@@ -119,3 +119,33 @@ def test_non_finite_elements_stay_visible(heom):
         r.close()
         assert not np.all(np.isfinite(gim[0]))
         assert np.all(np.isfinite(gre[15:])) and np.all(np.isfinite(gim[15:]))  # level 2: no link to the root
+
+
+@pytest.mark.parametrize("sites,K,D,precision", [(1, 1, 3, "fp64"), (2, 0, 6, "fp32_mixed"), (7, 1, 3, "fp32_mixed"),
+                                                 (7, 1, 2, "fp64"), (9, 1, 1, "fp32_mixed"), (16, 0, 3, "fp32_mixed"),
+                                                 (23, 0, 2, "fp32_mixed"), (23, 0, 2, "fp64"), (5, 2, 2, "fp64")])
+def test_column_whole_steps_equal_stages(heom, sites, K, D, precision):
+    """Column-0 runs: whole steps per launch and single stages (kernel timing on) give the same bits in every record
+    and ADO; FP64 within 1e-12 of the oracle, mixed correlations within 1e-5 of it (K = 2: up to six records per
+    state, D = 1: no FP32 body)."""
+    rng = np.random.default_rng(1803400 + sites)
+    H = np.diag(rng.uniform(0.0, 400.0, sites)) + np.triu(rng.normal(0.0, 40.0, (sites, sites)), 1)
+    s = wl.System(f"{sites} sites", H + np.triu(H, 1).T, list(range(sites)), [35.0] * sites, [60.0] * sites,
+                  [300.0] * sites, K=K, D=D)
+    p = wl.dipole_runs(s, wl.unit_dipoles(rng, sites), 0.5, 23, "col")[0]
+    m, ore, oim, oobs = oracle_propagate(p, p.n_steps, stride=5)
+    got = []
+    for timing in (False, True):
+        r = heom.Run(p.system, p.rho0_re, p.rho0_im, precision=precision, w=p.w, max_records=8)
+        assert r.layout() == 1
+        r.set_timing(timing)
+        r.propagate(p.dt_fs, p.n_steps, 5)
+        got.append((r.get_ados(0, r.n_ado), r.observables()))
+        r.close()
+    assert np.array_equal(got[0][1], got[1][1])
+    assert np.array_equal(got[0][0][0], got[1][0][0]) and np.array_equal(got[0][0][1], got[1][0][1])
+    N = sites + 1
+    tol = (1e-12 if precision == "fp64" else 1e-5) * max(1.0, np.max(np.abs(oobs)))
+    assert np.max(np.abs(got[0][1][:, :N + 4] - oobs)) <= tol
+    if precision == "fp64":
+        assert np.max(np.abs(got[0][0][0] + 1j * got[0][0][1] - (ore + 1j * oim))) <= tol
