@@ -189,6 +189,17 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
   const int Ep = c.Ep;
   const double ch = a.ch;
 
+  // the lane's pairs (i <= jj, numbered row by row): i << 8 | jj
+  int pairs[(N * (N + 1) / 2 + 31) / 32];
+#pragma unroll
+  for (int t0 = 0; t0 < N * (N + 1) / 2; t0 += 32) {
+    const int t = t0 + lane;
+    int i = 0;
+#pragma unroll
+    for (int w = 1; w < N; ++w) i += t >= w * N - w * (w - 1) / 2;
+    pairs[t0 / 32] = i << 8 | (t - (i * N - i * (i - 1) / 2) + i);
+  }
+
   const int n_chunks = (c.u_end - c.u_begin + G - 1) / G;
   const int nwarps = gridDim.x * S::WARPS;
   for (int chn = blockIdx.x * S::WARPS + warp; chn < n_chunks; chn += nwarps) {
@@ -221,11 +232,11 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
       const int ad = col / C, rem = col - ad * C;
       const int p = rem / N, j = rem - p * N;
       const bool act = ad < cnt;
-      double2 zc[N];
+      double zc[N];  // column j of the part that H multiplies: Im s for Q_re, Re s for Q_im
       if (act) {
-        const double2 *zt = zin + (int64_t)(u0 + ad) * Ep + j;
+        const double *zt = reinterpret_cast<const double *>(zin + (int64_t)(u0 + ad) * Ep + j) + (1 - p);
 #pragma unroll
-        for (int k = 0; k < N; ++k) zc[k] = zt[k * N];
+        for (int k = 0; k < N; ++k) zc[k] = zt[2 * k * N];
       }
       col_wait_all();
       __syncwarp();
@@ -235,19 +246,19 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
         // p = 0: Q_re = H Im s + coef Re s;  p = 1: Q_im = -H Re s + coef Im s
         int key = 0;
 #pragma unroll
-        for (int k = 0; k < N; ++k) key = max(key, fx_key(p ? zc[k].x : zc[k].y));
+        for (int k = 0; k < N; ++k) key = max(key, fx_key(zc[k]));
         double *qs = qring + (ad % S::RING) * 2 * E + p * E;
         if (fx_ok(a.ex << 20, key)) {
           const int ex = fx_exp(key);
           int2 src[N];
 #pragma unroll
-          for (int k = 0; k < N; ++k) src[k] = fx_split(p ? col_neg(zc[k].x) : zc[k].y, ex, kColBits);
+          for (int k = 0; k < N; ++k) src[k] = fx_split(p ? col_neg(zc[k]) : zc[k], ex, kColBits);
           const double *cf = coef + ad * N;
           const double gd = gh[ad];
           const int e2 = key ? a.ex - 2042 - 2 * kColBits + ex : 0;  // a zero column: any scale in range
           const double *zo = reinterpret_cast<const double *>(zin + (int64_t)(u0 + ad) * Ep + j) + p;  // own part
-          // rows in a loop: unrolled over them (2700 instructions) the code outgrew the instruction cache and the kernel
-          // took 20 ms at the LHCII size
+          // Rows in a loop, two at a time: unrolled over all of them (2700 instructions) the code outgrew the instruction
+          // cache and the kernel took 20 ms at the LHCII size; one at a time 8.8 ms, two 8.4 (5 CTAs per SM: 9.4)
 #pragma unroll 2
           for (int i = 0; i < N; ++i) {
             const double own = zo[2 * i * N], ci = i == j ? gd : cf[i];
@@ -292,11 +303,7 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
           for (int t0 = 0; t0 < PR; t0 += 32) {
             const int t = t0 + lane;
             if (t < PR) {
-              // row of pair t: the largest i with i N - i (i - 1) / 2 <= t
-              int i = 0;
-#pragma unroll
-              for (int w = 1; w < N; ++w) i += t >= w * N - w * (w - 1) / 2;
-              const int jj = t - (i * N - i * (i - 1) / 2) + i;
+              const int i = pairs[t0 / 32] >> 8, jj = pairs[t0 / 32] & 255;
               double2 yr = make_double2(0, 0);
               if (has_y) yr = y2[i * N + jj];
               const double rx = qs[i * N + jj] + qs[jj * N + i];  // Re R symmetric, Im R antisymmetric
