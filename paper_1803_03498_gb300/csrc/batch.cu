@@ -32,6 +32,15 @@ static void set_batch_schedule(VecBatchArgs &x, const std::vector<int64_t> &ados
   x.cpw = sc.chunks_per_warp;
 }
 
+// H and the terminator of a run into its descriptor, in the precision of the launch (vec_desc_H).
+template <typename T>
+static void fill_desc_H(T *H, const heom_run *r) {
+  for (int a = 0; a < r->n; ++a) {
+    for (int c = 0; c < r->n; ++c) H[a * kMaxStates + c] = (T)r->H[(size_t)a * r->n + c];
+    H[kMaxStates * kMaxStates + a] = (T)r->term[a];
+  }
+}
+
 struct heom_batch {
   std::vector<heom_run *> runs;
   std::vector<cudaStream_t> pool;
@@ -148,9 +157,8 @@ extern "C" int heom_batch_create(heom_run *const *runs, int n_runs, double dt_fs
           d.c.u_end = (part == 0 && !fp64) ? r->u_split : (int)r->n_ado;
           if (part == 0 && fp64) d.c.u_end = 0;  // FP64 runs: one part
           d.ch = chs[st];
-          for (int a = 0; a < r->n; ++a)
-            for (int c2 = 0; c2 < r->n; ++c2) d.H[a * kMaxStates + c2] = r->H[a * r->n + c2];
-          for (int a = 0; a < r->n; ++a) d.term[a] = r->term[a];
+          if (part == 1 && !fp64) fill_desc_H(reinterpret_cast<float *>(d.H), r);
+          else fill_desc_H(d.H, r);
           ba[st * 2 + part].d[q] = r->desc_dev + st * 2 + part;
           if (st == 0) ados[part == 0 ? 1 : 0].push_back(std::max(0, d.c.u_end - d.c.u_begin));
         }

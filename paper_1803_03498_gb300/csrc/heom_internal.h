@@ -133,8 +133,8 @@ HEOM_DECLARE_VEC(4)
 struct VecRunDesc {
   StageCommon c;
   double ch;
-  double H[kMaxStates * kMaxStates];  // row-major, stride kMaxStates (shifted H, rad/fs)
-  double term[kMaxStates];
+  // row-major H, stride kMaxStates (shifted, rad/fs), then Delta per state: doubles, or floats for an FP32 body
+  double H[kMaxStates * kMaxStates + kMaxStates];
 };
 constexpr int kBatchMaxRuns = 1024;   // runs per batched launch (kernel-parameter space)
 struct VecBatchArgs {

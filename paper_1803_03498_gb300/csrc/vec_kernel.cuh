@@ -239,6 +239,13 @@ __global__ void __launch_bounds__(kVecWarps * 32) vec_stage_kernel(const __grid_
   for (int sp = gw; sp < n_steps; sp += nw) vec_step<N, CT, BT, G>(c, hrow, h00, term_i, a.ch, sp, lane, ws);
 }
 
+// H and the terminator of a batched run's descriptor in the precision of the launch (batch.cu writes them so: 15
+// conversions per lane and warp step kept the FP64 pipe busy).
+template <typename CT>
+__device__ __forceinline__ const CT *vec_desc_H(const VecRunDesc *d) {
+  return reinterpret_cast<const CT *>(d->H);
+}
+
 // Many runs of the same N in one launch (ragged batches): run k's warp steps (of vec_group(N, G)
 // chunks each) are the launch's steps [chunk0[k], chunk0[k+1]); its stage arguments sit in its own
 // workspace (d[k]).
@@ -253,7 +260,10 @@ __global__ void __launch_bounds__(kVecWarps * 32) vec_batch_kernel(const __grid_
   const int64_t total = a.chunk0[a.nruns];
   __shared__ VecWarpSmem<CT, vec_group(N, G)> wsm[kVecWarps];
   VecWarpSmem<CT, vec_group(N, G)> &ws = wsm[threadIdx.x >> 5];
-  int k = 0;
+  int cur = -1;  // the run whose arguments are in registers: a warp's next step is mostly of the same one
+  StageCommon c;
+  CT hrow[N];
+  CT h00 = 0, term_i = 0, ch = 0;
   for (int64_t g = gw; g < total; g += nw) {
     int lo = 0, hi = a.nruns - 1;  // the run holding global chunk g
     while (lo < hi) {
@@ -261,16 +271,19 @@ __global__ void __launch_bounds__(kVecWarps * 32) vec_batch_kernel(const __grid_
       if (a.chunk0[mid] <= g) lo = mid;
       else hi = mid - 1;
     }
-    k = lo;
-    const VecRunDesc *d = a.d[k];
-    const StageCommon c = d->c;  // by value: registers, not reloads after the chunk's stores
-    CT hrow[N];
+    if (lo != cur) {
+      cur = lo;
+      const VecRunDesc *d = a.d[cur];
+      c = d->c;
+      const CT *H = vec_desc_H<CT>(d), *term = H + kMaxStates * kMaxStates;
 #pragma unroll
-    for (int b = 0; b < N; ++b) hrow[b] = lane_ok ? (CT)__ldg(&d->H[li * kMaxStates + b]) : (CT)0;
-    const CT h00 = (CT)__ldg(&d->H[0]), term_i = lane_ok ? (CT)__ldg(&d->term[li]) : (CT)0;
-    vec_step<N, CT, BT, G>(c, hrow, h00, term_i, (CT)__ldg(&d->ch), (int)(g - a.chunk0[k]), lane, ws);
+      for (int b = 0; b < N; ++b) hrow[b] = lane_ok ? __ldg(&H[li * kMaxStates + b]) : (CT)0;
+      h00 = __ldg(&H[0]);
+      term_i = lane_ok ? __ldg(&term[li]) : (CT)0;
+      ch = (CT)__ldg(&d->ch);
+    }
+    vec_step<N, CT, BT, G>(c, hrow, h00, term_i, ch, (int)(g - a.chunk0[cur]), lane, ws);
   }
-  (void)k;
 }
 
 template <int N, typename CT, typename BT, int G>
