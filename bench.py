@@ -277,7 +277,8 @@ def fp64_and_gate(prop, gate_steps, warmup, ws, clocks):
                         "peak_basis": basis,
                         "flops": "4 N^3 per ADO (Hermitian form: H s only, s H = (H s)^dagger) + 8 N^2 "
                                  "+ 8 (N-1) per up link + 8 (2N-1) per down link",
-                        "kernel": "stage_col_kernel<14> (column form, FP64)", "avg_launch_ms": avg, "schedule": sched},
+                        "kernel": "stage_col_kernel<14> (column form, FP64; the commutator runs in exact integers, so the "
+                                  "FP64 pipe's peak does not bound these flops)", "avg_launch_ms": avg, "schedule": sched},
            "clocks": clk}
     gate = {"steps": gate_steps, "records": gate_steps + 1, "max_pop_err": pop_err, "bar": 1e-6,
             "pass": pop_err <= 1e-6,
@@ -370,7 +371,7 @@ def time_batch(steps=20, per_launch=10):
 
 def time_field(steps=40, warmup=3, sm_mhz=None):
     """Pump-pulse propagation of the FMO-like two-exciton space (7 sites: 29 states, K = 1, D = 4:
-    3060 ADOs of 29 x 29) on the general stage kernel: classic four-copy RK4 with H(t) at each stage
+    3060 ADOs of 29 x 29) on the element kernels: classic four-copy RK4 with H(t) at each stage
     time.  Device-timed steps; per-launch kernel time of the body launches; algorithmic flops per
     ADO-RHS evaluation 16 N^3 (complex H(t)) + 8 N^2 + 8 per link record of each coupled state."""
     import torch
@@ -413,7 +414,7 @@ def time_field(steps=40, warmup=3, sm_mhz=None):
             n_sm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
             peak, basis = fp64_peak_tflops(sm_mhz, n_sm)
             leg["roofline"] = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                               "frac": ach / peak, "peak_basis": basis, "kernel": "gen_stage_kernel<double,double>"}
+                               "frac": ach / peak, "peak_basis": basis, "kernel": "el_stage_kernel<double,double> (commutator in integers)"}
         out[precision] = leg
     return out
 

@@ -70,8 +70,8 @@ typedef struct heom_run heom_run;
  * time_dependent: 1 reserves a fourth state copy so that the run can take a laser field
  *   (heom_run_set_field) and be propagated by classic four-copy RK4 with H(t) at each stage time.
  * Runs with a bath_mask, with time_dependent = 1 or with more than 24 states (up to 32, e.g. the
- * 29 states of a 7-site two-exciton space) use the general stage kernel; all others use the
- * specialised ones.
+ * 29 states of a 7-site two-exciton space) use the element kernels in their general form; all others use
+ * the specialised ones.
  * All pointers are read during the call only (copied).
  */
 typedef struct {
@@ -148,7 +148,7 @@ int heom_bath_modes(const heom_system *sys, double *gamma, double *c, double *la
 /*
  * heom_run_bytes -- device workspace bytes a run of this system, hierarchy and precision needs,
  * including room for max_records observable records.  The hierarchy's n_modes must equal
- * n_baths * (n_matsubara + 1).  Supported: 1 <= n_states <= 32 (above 24 on the general stage kernel).
+ * n_baths * (n_matsubara + 1).  Supported: 1 <= n_states <= 32 (above 24 in the element kernels' general form).
  */
 int heom_run_bytes(const heom_system *sys, const heom_hier *h, int precision, int64_t max_records,
                    size_t *bytes);
@@ -166,7 +166,7 @@ int heom_run_bytes(const heom_system *sys, const heom_hier *h, int precision, in
  * heom_run_destroy.  Mixed-precision runs also own one library stream and two events: each stage's
  * small FP64 head launch runs there, forked from and joined back into the caller's stream, so that
  * it overlaps the body launch (work enqueued on the caller's stream stays ordered).  The bath
- * coefficients follow sys->decomposition (Matsubara or Pade).  Runs on the general stage kernel
+ * coefficients follow sys->decomposition (Matsubara or Pade).  General runs
  * (bath_mask, time_dependent or more than 24 states) always use the matrix layout.
  */
 int heom_run_create(const heom_system *sys, const heom_hier *h, int precision, int64_t max_records,
@@ -178,7 +178,10 @@ int heom_run_destroy(heom_run *r);
  * heom_propagate -- advance the whole hierarchy by n_steps steps of classic RK4 with step dt_fs
  * (four evaluations of the right-hand side of Eq. HEOM per step).  Every obs_stride steps (0 =
  * never) one observable record of sigma_0 is appended after the step.  Enqueued on the run's
- * stream; does not block.  Errors: HEOM_E_ARG (dt_fs <= 0, n_steps < 0, dt_fs times the fastest
+ * stream; does not block.  Small hierarchies advance many steps per (cooperative) launch, whose CTAs meet
+ * at a barrier after every stage (bounded: HEOM_E_TIMEOUT from heom_observables if it gave up); with kernel
+ * timing on, under stream capture, or in a context with too few SMs for the launch, every stage is a launch
+ * of its own, with the same results.  Errors: HEOM_E_ARG (dt_fs <= 0, n_steps < 0, dt_fs times the fastest
  * decay rate D * max gamma above 2.5, where RK4 is no longer stable), HEOM_E_NOMEM (the records
  * would overflow max_records), HEOM_E_CUDA.
  */
@@ -258,7 +261,8 @@ int heom_run_info(const heom_run *r, int64_t *n_ado, int *n_states, int *n_modes
  */
 int heom_run_layout(const heom_run *r);
 
-/* Kernel launches the library enqueued for this run since creation (all kinds). */
+/* Kernel launches the library enqueued for this run since creation (all kinds; a launch of many steps counts
+ * once). */
 int64_t heom_run_launches(const heom_run *r);
 
 /*
@@ -311,7 +315,8 @@ int heom_batch_destroy(heom_batch *b);
  * a real H, no laser field, at most 200,000 ADOs) of equal n_states advance in work-list launches:
  * one launch per RK4 stage and part (FP64 head, FP32 body) covers every such run of that size, each
  * run's stage arguments staged from its own workspace, so many small requests cost a few launches
- * per step instead of eight each.  Other runs launch on their own, on the same stream.  Everything is
+ * per step instead of eight each.  Small FP64 runs share launches of many steps (as heom_propagate), ahead of
+ * the others.  Other runs launch on their own, on the same stream.  Everything is
  * enqueued on cuda_stream (the launches of different sizes on library-created streams forked from and
  * joined back into it, with its priority), ordered after work already enqueued on each run's stream, and later work
  * on each run's stream is ordered after it; the call does not block, except that writing a run's

@@ -135,6 +135,10 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       small_steps.push_back(n_steps[i]);
     }
     if (!small.empty()) rc = el_propagate(small.data(), (int)small.size(), h, small_steps.data(), obs_stride, gs);
+    if (rc == kElNoRoom) {
+      rc = HEOM_OK;
+      done.assign(n_runs, false);
+    }
   }
   // Each size class gets a stream of its own for the whole call (forked from and joined back into the
   // caller's stream): the classes' launch chains run side by side, while the stages of one class

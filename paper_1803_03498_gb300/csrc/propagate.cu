@@ -104,7 +104,7 @@ int heom::launch_head(heom_run *r, StageCommon c, double ch, cudaStream_t s) {
   c.occ_pct = r->sched[1].occupancy_pct;
   c.cpw = r->sched[1].chunks_per_warp;
   const int rc = r->vec ? launch_stage_vec(2, c, ch, r->term.data(), r->H.data(), s, r->sm_count)
-                        : launch_el_stage(2, el_args(r, c, ch), s, r->sm_count);
+                        : launch_el_stage(2, el_args(r, c, ch), nullptr, s, r->sm_count);
   if (rc) return HEOM_E_CUDA;
   ++r->launches;
   return HEOM_OK;
@@ -125,7 +125,7 @@ int heom::launch_body(heom_run *r, StageCommon c, double ch, cudaStream_t s) {
   } else if (fp64) {
     if (el_small(r) || !r->herm || r->cplx_h) rc = 1;
     else rc = launch_stage_col(c, ch, r->term.data(), r->H.data(), s, r->sm_count);
-    if (rc == 1) rc = launch_el_stage(0, el_args(r, c, ch), s, r->sm_count);
+    if (rc == 1) rc = launch_el_stage(0, el_args(r, c, ch), nullptr, s, r->sm_count);
   } else {
     if (r->precision == HEOM_SPLIT_TF32 && r->herm && !r->cplx_h) {  // tensor-core commutator
       rc = launch_stage_tc_a(c, ch, r->term.data(), r->H.data(), s, r->sm_count);
@@ -157,6 +157,7 @@ static int run_stage_gen(heom_run *r, StateView zin, StateView b1, StateView o1,
   a.y2 = b2;
   a.out2 = o2;
   a.c2 = c2;
+  const double *mup = r->has_field ? r->mup.data() : nullptr;
   const bool fp64 = r->precision == HEOM_FP64;
   cudaStream_t hs = r->stream;
   int rc;
@@ -166,7 +167,7 @@ static int run_stage_gen(heom_run *r, StateView zin, StateView b1, StateView o1,
     ah.c.u_begin = 0;
     ah.c.u_end = r->u_split;
     ah.c.occ_pct = r->sched[1].occupancy_pct;
-    if (launch_el_stage(2, ah, hs, r->sm_count)) return HEOM_E_CUDA;
+    if (launch_el_stage(2, ah, mup, hs, r->sm_count)) return HEOM_E_CUDA;
     ++r->launches;
   }
   a.c.u_begin = fp64 ? 0 : r->u_split;
@@ -174,7 +175,7 @@ static int run_stage_gen(heom_run *r, StateView zin, StateView b1, StateView o1,
   a.c.occ_pct = r->sched[0].occupancy_pct;
   if (a.c.u_end > a.c.u_begin) {
     if ((rc = timed_begin(r))) return rc;
-    if (launch_el_stage(fp64 ? 0 : 1, a, r->stream, r->sm_count)) return HEOM_E_CUDA;
+    if (launch_el_stage(fp64 ? 0 : 1, a, mup, r->stream, r->sm_count)) return HEOM_E_CUDA;
     ++r->launches;
     if ((rc = timed_end(r, r->bytes_stage_y))) return rc;
   }
@@ -271,9 +272,12 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
     }
     return HEOM_OK;
   }
-  if (n_steps > 0 && el_small(r) && !r->timing && !capturing(r->stream))
-    return el_propagate(&r, 1, h, &n_steps, obs_stride, r->stream);
-  if (n_steps > 0 && col_small(r) && !r->timing && !capturing(r->stream)) return col_propagate(r, h, n_steps, obs_stride, r->stream);
+  if (n_steps > 0 && !r->timing && !capturing(r->stream) && (el_small(r) || col_small(r))) {
+    // whole steps per launch; a captured or timed call, or a context too small for the launch, goes stage by stage
+    const int rc = r->vec ? col_propagate(r, h, n_steps, obs_stride, r->stream)
+                          : el_propagate(&r, 1, h, &n_steps, obs_stride, r->stream);
+    if (rc != kElNoRoom) return rc;
+  }
   for (int64_t s = 0; s < n_steps; ++s) {
     int rc;
     if ((rc = run_stage(r, r->y, r->y, r->zA, h / 4))) return rc;
@@ -303,7 +307,8 @@ extern "C" int heom_observables(heom_run *r, double *out, int64_t cap_records, i
     return HEOM_E_BOUNDS;
   }
   if (err_flag) {
-    set_error("heom_observables: a device-side wait of the tensor-core stage kernel gave up (its results are invalid)");
+    set_error("heom_observables: a bounded device-side wait gave up (the tensor-core kernel's, or the barrier of a launch of whole "
+              "steps; the run's results are invalid)");
     return HEOM_E_TIMEOUT;
   }
   int64_t cnt = cnt_err[0];

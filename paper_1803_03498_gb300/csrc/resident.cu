@@ -38,7 +38,7 @@ int fit_ados(int n, int pitch, int pairs, size_t real_bytes, bool general, size_
 }
 
 template <typename CT, typename BT, bool CPLX>
-int launch_stage_kind(const ElStageArgs &a, cudaStream_t st, int sm_count) {
+int launch_stage_kind(const ElStageArgs &a, const double *mup, cudaStream_t st, int sm_count) {
   const auto kern = el_stage_kernel<CT, BT, sizeof(CT) == 8 ? kElFixed : kElGeneral, CPLX>;
   static std::atomic<bool> ready{false};
   if (!ready) {
@@ -64,7 +64,10 @@ int launch_stage_kind(const ElStageArgs &a, cudaStream_t st, int sm_count) {
   }
   const int per_sm = std::max(1, std::min((int)by_regs, (int)((227u << 10) / (smem + 1024))));
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(units, (int64_t)sched_ctas(per_sm, c.occ_pct) * sm_count));
-  kern<<<grid, kElThreads, smem, st>>>(a);
+  ElMup<CPLX> m{};
+  if constexpr (CPLX)
+    if (mup) std::copy(mup, mup + (size_t)c.n * c.n, m.v);
+  kern<<<grid, kElThreads, smem, st>>>(a, m, mup != nullptr);
   e = cudaGetLastError();
   if (e == cudaSuccess) return 0;
   set_error(std::string("element stage kernel launch: ") + cudaGetErrorString(e));
@@ -107,7 +110,7 @@ int launch_lean(const ElStageArgs &a, cudaStream_t st, int sm_count) {
 }
 }  // namespace
 
-int launch_el_stage(int kind, const ElStageArgs &in, cudaStream_t st, int sm_count) {
+int launch_el_stage(int kind, const ElStageArgs &in, const double *mup, cudaStream_t st, int sm_count) {
   ElStageArgs a = in;
   const StageCommon &c = a.c;
   const int n_ado = c.u_end - c.u_begin;
@@ -122,14 +125,14 @@ int launch_el_stage(int kind, const ElStageArgs &in, cudaStream_t st, int sm_cou
   a.apu = std::max(1, std::min(2 * kElThreads / P, fit_ados(c.n, pitch, P, rb, true, kElSmemMax / 2)));
   a.apu = std::max(1, std::min(a.apu, n_ado / (2 * sm_count)));
   if (n_ado < 2 * sm_count) a.splits = std::max(1, std::min(2 * sm_count / n_ado, P / 64));
-  const bool cplx = c.cplx_h || a.k.mup;
+  const bool cplx = c.cplx_h || mup;
   switch (kind) {
-    case 0: return cplx ? launch_stage_kind<double, double, true>(a, st, sm_count)
-                        : launch_stage_kind<double, double, false>(a, st, sm_count);
-    case 1: return cplx ? launch_stage_kind<float, float, true>(a, st, sm_count)
-                        : launch_stage_kind<float, float, false>(a, st, sm_count);
-    default: return cplx ? launch_stage_kind<double, float, true>(a, st, sm_count)
-                         : launch_stage_kind<double, float, false>(a, st, sm_count);
+    case 0: return cplx ? launch_stage_kind<double, double, true>(a, mup, st, sm_count)
+                        : launch_stage_kind<double, double, false>(a, mup, st, sm_count);
+    case 1: return cplx ? launch_stage_kind<float, float, true>(a, mup, st, sm_count)
+                        : launch_stage_kind<float, float, false>(a, mup, st, sm_count);
+    default: return cplx ? launch_stage_kind<double, float, true>(a, mup, st, sm_count)
+                         : launch_stage_kind<double, float, false>(a, mup, st, sm_count);
   }
 }
 
@@ -162,18 +165,18 @@ int launch_head_list(const HeadList &in, cudaStream_t st, int sm_count) {
 
 static const char kElTag = 0;  // desc_owner of runs whose descriptor area holds an ElRunDesc
 
-static size_t desc_bytes(int n) { return 512 + ((size_t)4 * n * n + n) * sizeof(double); }
+static size_t desc_bytes(int n) { return 512 + ((size_t)3 * n * n + n) * sizeof(double); }
 // The work-list arguments of the four stages follow (grouped runs: at most kMaxStates states).
-constexpr size_t kGroupArgsAt = (512 + (4 * kMaxStates * kMaxStates + kMaxStates) * sizeof(double) + 15) & ~(size_t)15;
+constexpr size_t kGroupArgsAt = (512 + (3 * kMaxStates * kMaxStates + kMaxStates) * sizeof(double) + 15) & ~(size_t)15;
 static_assert(kGroupArgsAt + 4 * sizeof(GroupArgs) <= 8 * sizeof(VecRunDesc), "the descriptor area holds them");
 static_assert(sizeof(ElRunDesc) <= 512, "descriptor header");
-static_assert(512 + (4 * kGenMaxStates * kGenMaxStates + kGenMaxStates) * sizeof(double) <= 8 * sizeof(VecRunDesc),
+static_assert(512 + (3 * kGenMaxStates * kGenMaxStates + kGenMaxStates) * sizeof(double) <= 8 * sizeof(VecRunDesc),
               "the descriptor area holds the element kernels' constants");
 
 ElConsts el_consts_of(const heom_run *r) {
   const double *k = reinterpret_cast<const double *>(reinterpret_cast<const char *>(r->desc_dev) + 512);
   const size_t E = (size_t)r->n * r->n;
-  return ElConsts{k, k + E, k + 2 * E, r->has_field ? k + 3 * E : nullptr, k + 4 * E};
+  return ElConsts{k, k + E, k + 2 * E, nullptr, k + 3 * E};
 }
 
 // The run's constants and descriptor (matrix layout), enqueued on the run's stream; the host data is pageable and
@@ -201,8 +204,7 @@ int el_upload(heom_run *r) {
   for (int i = 0; i < r->n; ++i)
     for (int j = 0; j < r->n; ++j)
       k[2 * E + (size_t)i * r->n + j] = r->gen ? r->T[(size_t)i * r->n + j] : i != j ? r->term[i] + r->term[j] : 0.0;
-  if (!r->mup.empty()) std::copy(r->mup.begin(), r->mup.end(), k + 3 * E);
-  std::copy(r->term.begin(), r->term.end(), k + 4 * E);
+  std::copy(r->term.begin(), r->term.end(), k + 3 * E);
   const cudaError_t e = cudaMemcpyAsync(r->desc_dev, buf.data(), buf.size(), cudaMemcpyHostToDevice, r->stream);
   if (e != cudaSuccess) return cuda_fail("stage constants upload", e);
   r->desc_owner = &kElTag;
@@ -311,6 +313,14 @@ bool el_small(const heom_run *r) {
   return r->precision == HEOM_FP32_MIXED && !r->cplx_h && r->u_split > 0 && cost32(r) <= kElMaxCost32;
 }
 
+// A cooperative launch that this context cannot hold at once (fewer SMs than the device has): nothing was enqueued, and
+// the caller launches stage by stage.
+static bool no_room(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return false;
+  cudaGetLastError();
+  return true;
+}
+
 // CTAs that an FP64 run needs to be kept (kRunKept).
 static int kept_ctas(const heom_run *r) {
   const int a = lean_ados(r->n, kLeanRunThreads);
@@ -405,6 +415,7 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
       void *args[] = {&L};
       cudaError_t ce = cudaLaunchCooperativeKernel((const void *)el_run_kernel<KIND>, dim3(cta), dim3(threads), args, smem, s);
       if (ce == cudaSuccess) ce = cudaGetLastError();
+      if (no_room(ce) && at == 0 && b0 == 0) return kElNoRoom;
       if (ce != cudaSuccess) return cuda_fail("element run kernel launch", ce);
       for (size_t q = 0; q < in.size(); ++q) {
         heom_run *r = runs[in[q]];
@@ -437,10 +448,14 @@ int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *ste
   }
   static int (*const fns[4])(heom_run *const *, int, double, const int64_t *, int64_t, cudaStream_t) = {
       propagate_kind<kRunKept>, propagate_kind<kRunMixed>, propagate_kind<kRunOther>, propagate_kind<kRunChunks>};
+  int n_done = 0;
   for (int kind = 0; kind < 4; ++kind) {
     if (rs[kind].empty()) continue;
     const int rc = fns[kind](rs[kind].data(), (int)rs[kind].size(), h, st[kind].data(), stride, s);
+    if (rc == kElNoRoom && n_done == 0) return rc;
+    if (rc == kElNoRoom) return cuda_fail("element run kernel launch", cudaErrorCooperativeLaunchTooLarge);
     if (rc != HEOM_OK) return rc;
+    ++n_done;
   }
   return HEOM_OK;
 }
@@ -505,6 +520,7 @@ int col_propagate(heom_run *r, double h, int64_t steps, int64_t stride, cudaStre
     void *args[] = {&a};
     cudaError_t e = cudaLaunchCooperativeKernel((const void *)col_run_kernel, dim3(a.hcta + c32), dim3(kColThreads), args, smem, s);
     if (e == cudaSuccess) e = cudaGetLastError();
+    if (no_room(e) && at == 0) return kElNoRoom;
     if (e != cudaSuccess) return cuda_fail("column run kernel launch", e);
     if (stride > 0) r->records_host += (r->steps_done + a.steps) / stride - r->steps_done / stride;
     r->steps_done += a.steps;

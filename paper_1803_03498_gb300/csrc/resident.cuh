@@ -101,6 +101,8 @@ struct ElSmem {
   CT *H, *Hi, *T, *term;
   C2 *tile;
   uint32_t *rng;     // [cnt][n] records of (ADO, state): begin | end << 16, relative to the chunk's first
+  int2 *rest;        // [cnt][pitch] the tiles' third limbs, Re and Im (fixed point)
+  int2 *hrest;       // [n][n] those of H and Im H
   int *key;          // [cnt][2] largest |Re|, |Im| of an ADO's tile: FP64 high word (fixed point)
   int *hkey;         // the same of H
   uint16_t *pair;    // element p of an ADO: i << 8 | j
@@ -114,6 +116,7 @@ __host__ __device__ inline size_t el_smem_bytes(int n, int cnt, int pitch, int p
   b = (b + 15) & ~(size_t)15;
   b += (size_t)cnt * pitch * 2 * real_bytes;
   b = (b + 15) & ~(size_t)15;
+  if (real_bytes == 8) b += (((size_t)cnt * pitch + (size_t)n * n) * 8 + 15) & ~(size_t)15;  // third limbs
   b += (size_t)cnt * n * 4 + (size_t)cnt * 8 + 16 + (size_t)pairs * 2;
   return (b + 15) & ~(size_t)15;
 }
@@ -135,6 +138,9 @@ __device__ __forceinline__ ElSmem<CT> el_carve(unsigned char *p, int n, int cnt,
   uintptr_t a = (reinterpret_cast<uintptr_t>(q) + 15) & ~(uintptr_t)15;
   s.tile = reinterpret_cast<C2 *>(a);
   a = (a + (size_t)cnt * pitch * sizeof(C2) + 15) & ~(uintptr_t)15;
+  s.rest = reinterpret_cast<int2 *>(a);
+  s.hrest = s.rest + (size_t)cnt * pitch;
+  if (sizeof(CT) == 8) a = (a + ((size_t)cnt * pitch + (size_t)n * n) * 8 + 15) & ~(uintptr_t)15;
   s.rng = reinterpret_cast<uint32_t *>(a);
   s.key = reinterpret_cast<int *>(s.rng + cnt * n);  // then the key of H
   s.pair = reinterpret_cast<uint16_t *>(s.key + 2 * cnt + 4);
@@ -187,10 +193,12 @@ __device__ __forceinline__ void el_fix_consts(const ElSmem<double> &s, int n) {
   key = __reduce_max_sync(0xffffffffu, key);
   if ((threadIdx.x & 31) == 0) atomicMax(s.hkey, key);
   __syncthreads();
-  const int ex = fx_exp(*s.hkey), lb = fx_bits(n, CPLX);
+  const int ex = fx_exp(*s.hkey);
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    reinterpret_cast<int2 *>(s.H)[e] = fx_split(s.H[e], ex, lb);
-    if (CPLX) reinterpret_cast<int2 *>(s.Hi)[e] = fx_split(s.Hi[e], ex, lb);
+    int2 rest = make_int2(0, 0);
+    reinterpret_cast<int2 *>(s.H)[e] = fx_split3(s.H[e], ex, rest.x);
+    if (CPLX) reinterpret_cast<int2 *>(s.Hi)[e] = fx_split3(s.Hi[e], ex, rest.y);
+    s.hrest[e] = rest;
   }
 }
 
@@ -221,12 +229,13 @@ __device__ __forceinline__ void el_fix_tiles(const ElSmem<double> &s, int n, int
     }
   }
   __syncthreads();
-  const int lb = fx_bits(n, CPLX);
   for (int e = threadIdx.x; e < total; e += blockDim.x) {
     const int la = e / pitch;
     const double2 z = s.tile[e];
-    const int2 a = fx_split(z.x, fx_exp(s.key[2 * la]), lb), b = fx_split(z.y, fx_exp(s.key[2 * la + 1]), lb);
+    int2 rest;
+    const int2 a = fx_split3(z.x, fx_exp(s.key[2 * la]), rest.x), b = fx_split3(z.y, fx_exp(s.key[2 * la + 1]), rest.y);
     reinterpret_cast<int4 *>(s.tile)[e] = make_int4(a.x, a.y, b.x, b.y);
+    s.rest[e] = rest;
   }
   __syncthreads();
 }
@@ -235,32 +244,35 @@ __device__ __forceinline__ void el_fix_tiles(const ElSmem<double> &s, int n, int
 template <bool CPLX>
 __device__ __forceinline__ void el_fix_comm(const ElSmem<double> &s, int n, int la, int pitch, int i, int j, double &cr,
                                             double &ci) {
-  const int lb = fx_bits(n, CPLX);
-  FxSum r, m;
+  FxLong r, m;
   const int4 *z = reinterpret_cast<const int4 *>(s.tile) + la * pitch;
   const int4 *zi = z + i * n, *zj = z + j;
+  const int2 *wi = s.rest + la * pitch + i * n, *wj = s.rest + la * pitch + j;
   const int2 *hi_ = reinterpret_cast<const int2 *>(s.H) + i * n, *hj = reinterpret_cast<const int2 *>(s.H) + j;
   const int2 *gi_ = reinterpret_cast<const int2 *>(s.Hi) + i * n, *gj = reinterpret_cast<const int2 *>(s.Hi) + j;
+  const int2 *vi = s.hrest + i * n, *vj = s.hrest + j;
 #pragma unroll 2
   for (int k = 0; k < n; ++k) {
     const int4 a = zj[k * n], b = zi[k];
-    const int2 h1 = hi_[k], h2 = hj[k * n];
-    r.add(h1.x, h1.y, a.x, a.y);
-    m.add(h1.x, h1.y, a.z, a.w);
-    const int nx = -h2.x, ny = -h2.y;
-    r.add(nx, ny, b.x, b.y);
-    m.add(nx, ny, b.z, b.w);
+    const int2 ar = wj[k * n], br = wi[k];
+    const int2 h1 = hi_[k], h2 = hj[k * n], r1 = vi[k], r2 = vj[k * n];
+    r.add(h1.x, h1.y, r1.x, a.x, a.y, ar.x);
+    m.add(h1.x, h1.y, r1.x, a.z, a.w, ar.y);
+    const int nx = -h2.x, ny = -h2.y, nr = -r2.x;
+    r.add(nx, ny, nr, b.x, b.y, br.x);
+    m.add(nx, ny, nr, b.z, b.w, br.y);
     if constexpr (CPLX) {
       const int2 g1 = gi_[k], g2 = gj[k * n];
-      r.add(-g1.x, -g1.y, a.z, a.w);
-      m.add(g1.x, g1.y, a.x, a.y);
-      r.add(g2.x, g2.y, b.z, b.w);
-      m.add(-g2.x, -g2.y, b.x, b.y);
+      r.add(-g1.x, -g1.y, -r1.y, a.z, a.w, ar.y);
+      m.add(g1.x, g1.y, r1.y, a.x, a.y, ar.x);
+      r.add(g2.x, g2.y, r2.y, b.z, b.w, br.y);
+      m.add(-g2.x, -g2.y, -r2.y, b.x, b.y, br.x);
     }
   }
-  const int eh = fx_exp(*s.hkey) - 2042 - 2 * lb;
-  cr = fx_double(r.total(lb), eh + fx_exp(s.key[2 * la]));
-  ci = fx_double(m.total(lb), eh + fx_exp(s.key[2 * la + 1]));
+  // a zero tile part (or H): any exponent in range
+  const int hk = *s.hkey, eh = fx_exp(hk) - 2042 - 3 * kFxLong, kx = s.key[2 * la], ky = s.key[2 * la + 1];
+  cr = r.value(hk && kx ? eh + fx_exp(kx) : 0);
+  ci = m.value(hk && ky ? eh + fx_exp(ky) : 0);
 }
 
 // The same by FP64 FMAs, from global memory.
@@ -677,19 +689,22 @@ __host__ __device__ __forceinline__ void row_dispatch(int n, F f) {
 }
 
 template <typename CT, typename BT, int FORM, bool CPLX>
-__global__ void __launch_bounds__(kElThreads, 2) el_stage_kernel(const __grid_constant__ ElStageArgs a) {
+__global__ void __launch_bounds__(kElThreads, 2) el_stage_kernel(const __grid_constant__ ElStageArgs a,
+                                                                 const __grid_constant__ ElMup<CPLX> m, int field) {
   extern __shared__ __align__(16) unsigned char el_sm[];
   constexpr bool OWN_HEAD = sizeof(CT) == 8 && sizeof(BT) == 4;
   const StageCommon &c = a.c;
   constexpr bool general = FORM != kElRowOrder;
   const ElSmem<CT> s = el_carve<CT>(el_sm, c.n, a.apu, OWN_HEAD ? c.E : c.Ep, el_pairs(c.n, c.herm), general);
-  el_consts<CT>(s, a.k, c.n, c.herm, general, a.gr, a.gi);
+  ElConsts k = a.k;
+  if constexpr (CPLX) k.mup = field ? m.v : nullptr;
+  el_consts<CT>(s, k, c.n, c.herm, general, a.gr, a.gi);
   __syncthreads();
   if constexpr (FORM == kElFixed) {
     el_fix_consts<CPLX>(s, c.n);
     __syncthreads();
   }
-  const ElStage g{c.zin, c.y, c.out, a.y2, a.out2, a.c1, a.c2, a.k, a.gr, a.gi};
+  const ElStage g{c.zin, c.y, c.out, a.y2, a.out2, a.c1, a.c2, k, a.gr, a.gi};
   bool built = false;
   el_units<CT, BT, FORM, CPLX, true>(s, c, g, ElPlan{a.apu, a.splits}, blockIdx.x, gridDim.x, built);
 }

