@@ -75,7 +75,11 @@ void cache_put(const std::array<int, 7> &k, const heom_schedule &s) {
 
 bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {  // e.g. the legacy stream beside another stream's capture
+    cudaGetLastError();                                // not a failure of the launches that follow
+    return true;
+  }
+  return cs != cudaStreamCaptureStatusNone;
 }
 
 
