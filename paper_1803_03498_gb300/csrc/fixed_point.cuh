@@ -8,7 +8,7 @@
 // floating-point slices.
 // What is cut off an element is below 2^(1 - 2 LB) of the largest one's binade (2^-57 or 2^-55; FP64 itself rounds
 // that element at 2^-54), and no sum rounds on the way.  Measured against 64-bit torch (relative 2-norm): four steps of
-// 1,344,904 ADOs of 14 x 14 from a site 1.7e-16, with FP64 FMAs 2.1e-16; 400 steps of 3060 ADOs of 7 x 7 1.6e-15
+// 1,344,904 ADOs of 14 x 14 from a site 1.7e-16 and 1.9e-16 on two inputs, with FP64 FMAs 2.1e-16 and 1.1e-16; 400 steps of 3060 ADOs of 7 x 7 1.6e-15
 // both.  Where elements of very different size share a scale and the small ones matter (general runs: Re and Im of
 // the two-exciton space under a pulse share it, populations beside weak coherences), the longer form below keeps 28
 // more bits of H, the tile and the sum: with the short one the error of ten steps grew from 1.2e-16 to 1.2e-15.
