@@ -205,7 +205,6 @@ struct ElStageArgs {
   StateView y2, out2;
   double c1, c2, gr, gi;
   int apu, splits;  // ADOs per unit, or (apu = 1) units per ADO (set by the launcher)
-  bool fixed;       // pair kernels: fixed-point commutator (set by the launcher)
   bool general;     // couplings with several states per bath, a laser field or more than 24 states
 };
 // kind as launch_stage_vec (the FP32 body only for general runs); mup: [n][n] M+ on the host, or NULL.

@@ -33,39 +33,43 @@ __host__ __device__ inline int lean_ados(int n, int threads) {
 __host__ __device__ inline bool lean_fixed(int n, int64_t ados) {
   return n >= 9 || (n >= 5 && ados * (n * (n + 1) / 2) >= 32768);
 }
+// The same for the head of a mixed run: its 1 + n_modes ADOs (at most 256) never reach the second line.
+__host__ __device__ constexpr bool lean_head_fixed(int n) { return n >= 9; }
 
 // Shared memory: limbs of H and of the tiles, T, scale keys (two sets), link ranges; and for resident CTAs the
 // coefficients of each thread's slots.
 struct LeanSmem {
   int4 *tile;      // [ados][n][n] Re hi, Re lo, Im hi, Im lo (fixed point) or the FP64 elements
+  int2 *rest;      // [ados][n][n] third limbs, Re and Im
   double2 *coef;   // [kLeanKept][threads] R (resident)
   double *T;       // [n][n]
   int2 *H;         // [n][n] limbs or FP64
+  int *hrest;      // [n][n] third limbs
   int *key;        // [2][2 ados]
   int *hkey;
   uint32_t *rng;   // [ados][n] begin | end << 16, relative to the ADO's first record
   unsigned char *end;
   int ados;        // ADOs per chunk
-  bool fixed;
 };
 __host__ __device__ inline size_t lean_smem_bytes(int n, int a, int kept_threads) {
   const size_t E = (size_t)n * n;
-  const size_t b = a * E * 16 + (size_t)kLeanKept * kept_threads * 16 + E * 16 + 16 * (size_t)a + 16 + 4 * (size_t)a * n;
+  const size_t b = a * E * 24 + (size_t)kLeanKept * kept_threads * 16 + E * 20 + 16 * (size_t)a + 16 + 4 * (size_t)a * n;
   return (b + 15) & ~(size_t)15;
 }
-__device__ __forceinline__ LeanSmem lean_carve(unsigned char *p, int n, int a, int kept_threads, bool fixed) {
+__device__ __forceinline__ LeanSmem lean_carve(unsigned char *p, int n, int a, int kept_threads) {
   const int E = n * n;
   LeanSmem s;
   s.tile = reinterpret_cast<int4 *>(p);
   s.coef = reinterpret_cast<double2 *>(s.tile + a * E);
-  s.T = reinterpret_cast<double *>(s.coef + kLeanKept * kept_threads);
+  s.rest = reinterpret_cast<int2 *>(s.coef + kLeanKept * kept_threads);
+  s.T = reinterpret_cast<double *>(s.rest + a * E);
   s.H = reinterpret_cast<int2 *>(s.T + E);
-  s.key = reinterpret_cast<int *>(s.H + E);
+  s.hrest = reinterpret_cast<int *>(s.H + E);
+  s.key = s.hrest + E;
   s.hkey = s.key + 4 * a;
   s.rng = reinterpret_cast<uint32_t *>(s.hkey + 4);
   s.end = p + lean_smem_bytes(n, a, kept_threads);
   s.ados = a;
-  s.fixed = fixed;
   return s;
 }
 
@@ -92,7 +96,8 @@ __device__ __forceinline__ LeanPair lean_pair(int n) {
   return p;
 }
 
-// H as limbs, T; synchronises the CTA.
+// H as limbs, T; synchronises the CTA.  FIXED: the commutator in fixed point (lean_fixed).
+template <bool FIXED>
 __device__ __forceinline__ void lean_consts(const LeanSmem &s, const ElConsts &k, int n) {
   if (threadIdx.x == 0) *s.hkey = 0;
   __syncthreads();
@@ -104,17 +109,18 @@ __device__ __forceinline__ void lean_consts(const LeanSmem &s, const ElConsts &k
   key = __reduce_max_sync(0xffffffffu, key);
   if ((threadIdx.x & 31) == 0) atomicMax(s.hkey, key);
   __syncthreads();
-  const int ex = fx_exp(*s.hkey), lb = fx_bits(n, false);
+  const int ex = fx_exp(*s.hkey);
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    if (s.fixed) s.H[e] = fx_split(k.H[e], ex, lb);
+    if (FIXED) s.H[e] = fx_split(k.H[e], ex, s.hrest[e]);
     else reinterpret_cast<double *>(s.H)[e] = k.H[e];
   }
   __syncthreads();
 }
 
 // Called by every thread of the CTA (z = 0 where a thread has no element).
+template <bool FIXED>
 __device__ __forceinline__ void lean_key(const LeanSmem &s, const LeanPair &p, int *key, double2 z) {
-  if (!s.fixed) return;
+  if (!FIXED) return;
   int kx = fx_key(z.x), ky = fx_key(z.y);
   if (p.whole) {
     kx = __reduce_max_sync(0xffffffffu, kx);
@@ -127,26 +133,47 @@ __device__ __forceinline__ void lean_key(const LeanSmem &s, const LeanPair &p, i
 }
 
 // The element and its mirror (conjugate) as limbs.
+template <bool FIXED>
 __device__ __forceinline__ void lean_limbs(const LeanSmem &s, const LeanPair &p, int n, const int *key, double2 z) {
-  if (!s.fixed) {
+  if constexpr (!FIXED) {
     double2 *t = reinterpret_cast<double2 *>(s.tile) + p.la * n * n;
     t[p.e] = z;
     if (p.i != p.j) t[p.em] = make_double2(z.x, -z.y);
-    return;
+  } else {
+    int2 w;
+    const int2 a = fx_split(z.x, fx_exp(key[2 * p.la]), w.x), b = fx_split(z.y, fx_exp(key[2 * p.la + 1]), w.y);
+    int4 *t = s.tile + p.la * n * n;
+    int2 *tw = s.rest + p.la * n * n;
+    t[p.e] = make_int4(a.x, a.y, b.x, b.y);
+    tw[p.e] = w;
+    if (p.i != p.j) {
+      t[p.em] = make_int4(a.x, a.y, -b.x, -b.y);
+      tw[p.em] = make_int2(w.x, -w.y);
+    }
   }
-  const int lb = fx_bits(n, false);
-  const int2 a = fx_split(z.x, fx_exp(key[2 * p.la]), lb), b = fx_split(z.y, fx_exp(key[2 * p.la + 1]), lb);
-  int4 *t = s.tile + p.la * n * n;
-  t[p.e] = make_int4(a.x, a.y, b.x, b.y);
-  if (p.i != p.j) t[p.em] = make_int4(a.x, a.y, -b.x, -b.y);
 }
 
-// -i (H z - z H)_ij - f z_ij; zin: the ADO's tile in global memory (read only where fixed point does not fit).
+// C = H z - z H of element (i, j) by FP64 FMAs, H and the ADO's tile z in global memory.
+__device__ __noinline__ double2 lean_fma_comm(const double *H, const double2 *z, int n, int i, int j) {
+  double ar = 0, ai = 0, br = 0, bi = 0;
+#pragma unroll 4
+  for (int k = 0; k < n; ++k) {
+    const double2 a = __ldcg(z + k * n + j), b = __ldcg(z + i * n + k);
+    const double h1 = H[i * n + k], h2 = H[k * n + j];
+    ar = fma(h1, a.x, ar);
+    ai = fma(h1, a.y, ai);
+    br = fma(b.x, h2, br);
+    bi = fma(b.y, h2, bi);
+  }
+  return make_double2(ar - br, ai - bi);
+}
+
+// -i (H z - z H)_ij - f z_ij; zin: the ADO's tile in global memory (read only where the FMA chain takes over).
+template <bool FIXED>
 __device__ __forceinline__ double2 lean_comm(const LeanSmem &s, const LeanPair &p, int n, const int *key, double2 z, double f,
                                              const double2 *zin, const ElConsts &kc) {
-  const int kx = key[2 * p.la], ky = key[2 * p.la + 1], hk = *s.hkey;
-  double cr, ci;
-  if (!s.fixed) {
+  double cr = 0, ci = 0;
+  if constexpr (!FIXED) {
     double ar = 0, ai = 0, br = 0, bi = 0;
     const double2 *zi = reinterpret_cast<const double2 *>(s.tile) + (p.la * n + p.i) * n;
     const double2 *zj = reinterpret_cast<const double2 *>(s.tile) + p.la * n * n + p.j;
@@ -163,27 +190,37 @@ __device__ __forceinline__ double2 lean_comm(const LeanSmem &s, const LeanPair &
     }
     cr = ar - br;
     ci = ai - bi;
-  } else if (fx_ok(hk, kx) && fx_ok(hk, ky)) {
-    FxSum r, m;
-    const int4 *zi = s.tile + (p.la * n + p.i) * n, *zj = s.tile + p.la * n * n + p.j;
-    const int2 *hi_ = s.H + p.i * n, *hj = s.H + p.j;
-#pragma unroll 2
-    for (int k = 0; k < n; ++k) {
-      const int4 a = *zj, b = zi[k];
-      const int2 h1 = hi_[k], h2 = *hj;
-      zj += n;
-      hj += n;
-      r.add(h1.x, h1.y, a.x, a.y);
-      m.add(h1.x, h1.y, a.z, a.w);
-      const int nx = -h2.x, ny = -h2.y;
-      r.add(nx, ny, b.x, b.y);
-      m.add(nx, ny, b.z, b.w);
-    }
-    const int lb = fx_bits(n, false), eh = fx_exp(hk) - 2042 - 2 * lb;
-    cr = fx_double(r.total(lb), eh + fx_exp(kx));
-    ci = fx_double(m.total(lb), eh + fx_exp(ky));
   } else {
-    el_fma_comm<false>(kc, zin, n, p.i, p.j, 0.0, 0.0, cr, ci);
+    const int kx = key[2 * p.la], ky = key[2 * p.la + 1], hk = *s.hkey;
+    int chain = 3;  // bits: Re C, Im C by FMAs
+    if (fx_ok(hk, kx) && fx_ok(hk, ky)) {
+      FxSum r, m;
+      const int4 *zi = s.tile + (p.la * n + p.i) * n, *zj = s.tile + p.la * n * n + p.j;
+      const int2 *wi = s.rest + (p.la * n + p.i) * n, *wj = s.rest + p.la * n * n + p.j;
+      const int2 *hi_ = s.H + p.i * n, *hj = s.H + p.j;
+      const int *vi = s.hrest + p.i * n, *vj = s.hrest + p.j;
+#pragma unroll 2
+      for (int k = 0; k < n; ++k) {
+        const int4 a = *zj, b = zi[k];
+        const int2 ar = *wj, br = wi[k], h1 = hi_[k], h2 = *hj;
+        const int r1 = vi[k], nx = -h2.x, ny = -h2.y, nr = -*vj;
+        zj += n;
+        wj += n;
+        hj += n;
+        vj += n;
+        r.add(h1.x, h1.y, r1, a.x, a.y, ar.x);
+        m.add(h1.x, h1.y, r1, a.z, a.w, ar.y);
+        r.add(nx, ny, nr, b.x, b.y, br.x);
+        m.add(nx, ny, nr, b.z, b.w, br.y);
+      }
+      chain = fx_finish(r, m, hk, kx, ky, cr, ci);
+    }
+    if (p.i == p.j) chain &= 2;  // Re C = 0 there and is not used
+    if (chain) {
+      const double2 x = lean_fma_comm(kc.H, zin, n, p.i, p.j);
+      if (chain & 1) cr = x.x;
+      if (chain & 2) ci = x.y;
+    }
   }
   return make_double2(fma(-f, z.x, ci), fma(-f, z.y, -cr));
 }
@@ -235,7 +272,7 @@ __device__ __forceinline__ void lean_ranges(const LeanSmem &s, const StageCommon
 }
 
 // Chunks first, first + stride, ... of one stage.
-template <typename BT>
+template <typename BT, bool FIXED>
 __device__ __forceinline__ void lean_chunks(const LeanSmem &s, const LeanPair &p, const StageCommon &c, double ch,
                                             const ElConsts &kc, int first, int stride) {
   constexpr bool OWN_HEAD = sizeof(BT) == 4;
@@ -261,7 +298,7 @@ __device__ __forceinline__ void lean_chunks(const LeanSmem &s, const LeanPair &p
     if (threadIdx.x < 2 * A) s.key[threadIdx.x] = 0;
     __syncthreads();
     lean_ranges<BT>(s, c, u0, 1, cnt);
-    lean_key(s, p, s.key, z);
+    lean_key<FIXED>(s, p, s.key, z);
     __syncthreads();
     LeanLinks l{0, 0, 0, 0};
     ElRec<double> rec[kLeanSlots];
@@ -276,11 +313,11 @@ __device__ __forceinline__ void lean_chunks(const LeanSmem &s, const LeanPair &p
         v[q] = make_double2(0, 0);
         if (q < l.nq && HEOM_IN_RANGE(c.err, rec[q].v, 0, c.n_ado)) v[q] = el_fetch<double, BT>(c.zin, c, rec[q].v, p.e);
       }
-      lean_limbs(s, p, n, s.key, z);
+      lean_limbs<FIXED>(s, p, n, s.key, z);
     }
     __syncthreads();
     if (!have) continue;
-    double2 r = lean_comm(s, p, n, s.key, z, f, zt, kc);
+    double2 r = lean_comm<FIXED>(s, p, n, s.key, z, f, zt, kc);
 #pragma unroll
     for (int q = 0; q < kLeanSlots; ++q)
       if (q < l.nq) lean_link(r, rec[q].re, rec[q].im, v[q], q < l.ni);
@@ -311,7 +348,7 @@ struct LeanState {
   bool have;
 };
 
-template <typename BT>
+template <typename BT, bool FIXED>
 __device__ __forceinline__ void lean_begin(LeanState &t, const LeanSmem &s, const LeanPair &p, const StageCommon &c, int first,
                                            int stride) {
   constexpr bool OWN_HEAD = sizeof(BT) == 4;
@@ -333,7 +370,7 @@ __device__ __forceinline__ void lean_begin(LeanState &t, const LeanSmem &s, cons
     t.f = __ldg(c.gsum + t.u) + s.T[p.e];
     t.recs = lean_recs<BT>(c, __ldg(c.link_off + t.u));
   }
-  lean_key(s, p, s.key, t.z);
+  lean_key<FIXED>(s, p, s.key, t.z);
   __syncthreads();
   if (t.have) {
     t.l = lean_links(s, p, n);
@@ -350,7 +387,7 @@ __device__ __forceinline__ void lean_begin(LeanState &t, const LeanSmem &s, cons
 }
 
 // One stage; the first of a step also takes y = z, and the last one leaves the step's result in z.
-template <typename BT>
+template <typename BT, bool FIXED>
 __device__ __forceinline__ void lean_step(LeanState &t, const LeanSmem &s, const LeanPair &p, const StageCommon &c, double ch,
                                           const ElConsts &kc, bool begins) {
   constexpr bool OWN_HEAD = sizeof(BT) == 4;
@@ -363,12 +400,12 @@ __device__ __forceinline__ void lean_step(LeanState &t, const LeanSmem &s, const
 #pragma unroll
     for (int q = 0; q < kLeanKept; ++q)
       if (q < t.l.nq) v[q] = el_fetch<double, BT>(c.zin, c, t.v[q], p.e);
-    lean_limbs(s, p, n, key, t.z);
+    lean_limbs<FIXED>(s, p, n, key, t.z);
   }
   if (threadIdx.x < 2 * A) next[threadIdx.x] = 0;
   __syncthreads();
   if (t.have) {
-    double2 r = lean_comm(s, p, n, key, t.z, t.f, el_own<double, BT, OWN_HEAD>(c.zin, c, t.u), kc);
+    double2 r = lean_comm<FIXED>(s, p, n, key, t.z, t.f, el_own<double, BT, OWN_HEAD>(c.zin, c, t.u), kc);
 #pragma unroll
     for (int q = 0; q < kLeanKept; ++q)
       if (q < t.l.nq) {
@@ -386,17 +423,17 @@ __device__ __forceinline__ void lean_step(LeanState &t, const LeanSmem &s, const
     __stcg(d + p.e, t.z);
     if (p.i != p.j) __stcg(d + p.em, make_double2(t.z.x, -t.z.y));
   }
-  lean_key(s, p, next, t.z);
+  lean_key<FIXED>(s, p, next, t.z);
 }
 
 // One stage of a range of ADOs.
-template <typename BT>
+template <typename BT, bool FIXED>
 __global__ void __launch_bounds__(kLeanThreads, 2) lean_stage_kernel(const __grid_constant__ ElStageArgs a) {
   extern __shared__ __align__(16) unsigned char el_sm[];
-  const LeanSmem s = lean_carve(el_sm, a.c.n, a.apu, 0, a.fixed);
-  lean_consts(s, a.k, a.c.n);
+  const LeanSmem s = lean_carve(el_sm, a.c.n, a.apu, 0);
+  lean_consts<FIXED>(s, a.k, a.c.n);
   const LeanPair p = lean_pair(a.c.n);
-  lean_chunks<BT>(s, p, a.c, a.c1, a.k, blockIdx.x, gridDim.x);
+  lean_chunks<BT, FIXED>(s, p, a.c, a.c1, a.k, blockIdx.x, gridDim.x);
 }
 
 }  // namespace heom

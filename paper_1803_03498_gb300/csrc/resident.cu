@@ -80,13 +80,13 @@ int launch_stage_kind(const ElStageArgs &a, const double *mup, cudaStream_t st, 
 bool lean_covers(int n, int herm, int cplx, bool general) { return herm && !cplx && !general && n <= kLeanMaxStates; }
 
 namespace {
-template <typename BT>
+template <typename BT, bool FIXED>
 int launch_lean(const ElStageArgs &a, cudaStream_t st, int sm_count) {
   static std::atomic<int> by_regs{0};
   cudaError_t e = cudaSuccess;
   if (by_regs == 0) {
     int ps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, lean_stage_kernel<BT>, kLeanThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, lean_stage_kernel<BT, FIXED>, kLeanThreads, 0);
     if (e != cudaSuccess || ps < 1) {
       set_error(std::string("pair stage kernel: occupancy query failed or zero blocks: ") + cudaGetErrorString(e));
       return -4;
@@ -97,12 +97,10 @@ int launch_lean(const ElStageArgs &a, cudaStream_t st, int sm_count) {
   ElStageArgs x = a;
   // fewer ADOs per CTA where there are not enough for every CTA slot
   x.apu = std::max(1, std::min(lean_ados(a.c.n, kLeanThreads), n_ado / (2 * sm_count)));
-  // the part of the run, not of the launch, decides (see lean_fixed)
-  x.fixed = lean_fixed(a.c.n, sizeof(BT) == 4 ? a.c.u_split : a.c.n_ado);
   const int chunks = (n_ado + x.apu - 1) / x.apu;
   const size_t smem = lean_smem_bytes(a.c.n, x.apu, 0);  // below 48 KB
   const int grid = std::max(1, std::min(chunks, sched_ctas(by_regs, a.c.occ_pct) * sm_count));
-  lean_stage_kernel<BT><<<grid, kLeanThreads, smem, st>>>(x);
+  lean_stage_kernel<BT, FIXED><<<grid, kLeanThreads, smem, st>>>(x);
   e = cudaGetLastError();
   if (e == cudaSuccess) return 0;
   set_error(std::string("pair stage kernel launch: ") + cudaGetErrorString(e));
@@ -115,8 +113,12 @@ int launch_el_stage(int kind, const ElStageArgs &in, const double *mup, cudaStre
   const StageCommon &c = a.c;
   const int n_ado = c.u_end - c.u_begin;
   if (n_ado <= 0) return 0;
-  if (kind != 1 && lean_covers(c.n, c.herm, c.cplx_h, a.general))
-    return kind == 0 ? launch_lean<double>(a, st, sm_count) : launch_lean<float>(a, st, sm_count);
+  if (kind != 1 && lean_covers(c.n, c.herm, c.cplx_h, a.general)) {
+    // the part of the run, not of the launch, decides (see lean_fixed)
+    const bool fixed = kind == 0 ? lean_fixed(c.n, c.n_ado) : lean_head_fixed(c.n);
+    if (kind == 0) return fixed ? launch_lean<double, true>(a, st, sm_count) : launch_lean<double, false>(a, st, sm_count);
+    return fixed ? launch_lean<float, true>(a, st, sm_count) : launch_lean<float, false>(a, st, sm_count);
+  }
   const size_t rb = kind == 1 ? 4 : 8;
   const int P = el_pairs(c.n, c.herm), pitch = kind == 2 ? c.E : c.Ep;
   // units of about two rounds of the CTA's threads; fewer ADOs than CTA slots (2 per SM) take smaller units, and
@@ -145,15 +147,16 @@ int launch_head_list(const HeadList &in, cudaStream_t st, int sm_count) {
   const size_t smem = lean ? lean_smem_bytes(L.n, L.apu, 0)
                            : el_smem_bytes(L.n, L.apu, L.n * L.n, el_pairs(L.n, L.herm), 8, true);
   if (lean) {
-    head_list_kernel<true><<<ctas, kElThreads, smem, st>>>(L);
+    if (lean_head_fixed(L.n)) head_list_kernel<true, true><<<ctas, kElThreads, smem, st>>>(L);
+    else head_list_kernel<true, false><<<ctas, kElThreads, smem, st>>>(L);
   } else {
     static std::atomic<bool> ready{false};
     if (!ready) {
-      const int rc = max_smem((const void *)head_list_kernel<false>, "head list kernel");
+      const int rc = max_smem((const void *)head_list_kernel<false, true>, "head list kernel");
       if (rc) return rc;
       ready = true;
     }
-    head_list_kernel<false><<<ctas, kElThreads, smem, st>>>(L);
+    head_list_kernel<false, true><<<ctas, kElThreads, smem, st>>>(L);
   }
   const cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) return 0;
@@ -327,11 +330,11 @@ static int kept_ctas(const heom_run *r) {
   return (int)((r->n_ado + a - 1) / a);
 }
 
-template <int KIND>
+template <int KIND, bool FIXED>
 static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
   static std::atomic<bool> ready{false};
   if (!ready) {
-    const int rc = max_smem((const void *)el_run_kernel<KIND>, "element run kernel");
+    const int rc = max_smem((const void *)el_run_kernel<KIND, FIXED>, "element run kernel");
     if (rc) return HEOM_E_CUDA;
     ready = true;
   }
@@ -413,7 +416,7 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
         }
       }
       void *args[] = {&L};
-      cudaError_t ce = cudaLaunchCooperativeKernel((const void *)el_run_kernel<KIND>, dim3(cta), dim3(threads), args, smem, s);
+      cudaError_t ce = cudaLaunchCooperativeKernel((const void *)el_run_kernel<KIND, FIXED>, dim3(cta), dim3(threads), args, smem, s);
       if (ce == cudaSuccess) ce = cudaGetLastError();
       if (no_room(ce) && at == 0 && b0 == 0) return kElNoRoom;
       if (ce != cudaSuccess) return cuda_fail("element run kernel launch", ce);
@@ -433,25 +436,32 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
 // Steps [done, done + steps[i]) of every run on stream s, as few launches as possible; the runs' counters
 // (steps_done, t_fs, records_host, launches) advance.
 int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
-  std::vector<heom_run *> rs[4];
-  std::vector<int64_t> st[4];
-  int need = 0;
+  // kRunKept, kRunMixed and kRunChunks without and with fixed point, then the others
+  constexpr int kForms = 7;
+  std::vector<heom_run *> rs[kForms];
+  std::vector<int64_t> st[kForms];
+  auto fixed = [](const heom_run *r) {
+    return r->precision == HEOM_FP64 ? lean_fixed(r->n, r->n_ado) : lean_head_fixed(r->n);
+  };
+  int need[2] = {0, 0};
   for (int i = 0; i < n_runs; ++i)
-    if (run_lean(runs[i]) && runs[i]->precision == HEOM_FP64) need += kept_ctas(runs[i]);
+    if (run_lean(runs[i]) && runs[i]->precision == HEOM_FP64) need[fixed(runs[i])] += kept_ctas(runs[i]);
   for (int i = 0; i < n_runs; ++i) {
-    const int kind = !run_lean(runs[i])                     ? kRunOther
-                     : runs[i]->precision != HEOM_FP64      ? kRunMixed
-                     : need <= 2 * runs[i]->sm_count ? kRunKept
-                                                            : kRunChunks;
-    rs[kind].push_back(runs[i]);
-    st[kind].push_back(steps[i]);
+    const bool fx = fixed(runs[i]);
+    const int form = !run_lean(runs[i])                     ? 6
+                     : runs[i]->precision != HEOM_FP64      ? 2 + fx
+                     : need[fx] <= 2 * runs[i]->sm_count ? 0 + fx
+                                                         : 4 + fx;
+    rs[form].push_back(runs[i]);
+    st[form].push_back(steps[i]);
   }
-  static int (*const fns[4])(heom_run *const *, int, double, const int64_t *, int64_t, cudaStream_t) = {
-      propagate_kind<kRunKept>, propagate_kind<kRunMixed>, propagate_kind<kRunOther>, propagate_kind<kRunChunks>};
+  static int (*const fns[kForms])(heom_run *const *, int, double, const int64_t *, int64_t, cudaStream_t) = {
+      propagate_kind<kRunKept, false>,  propagate_kind<kRunKept, true>,   propagate_kind<kRunMixed, false>, propagate_kind<kRunMixed, true>,
+      propagate_kind<kRunChunks, false>, propagate_kind<kRunChunks, true>, propagate_kind<kRunOther, true>};
   int n_done = 0;
-  for (int kind = 0; kind < 4; ++kind) {
-    if (rs[kind].empty()) continue;
-    const int rc = fns[kind](rs[kind].data(), (int)rs[kind].size(), h, st[kind].data(), stride, s);
+  for (int form = 0; form < kForms; ++form) {
+    if (rs[form].empty()) continue;
+    const int rc = fns[form](rs[form].data(), (int)rs[form].size(), h, st[form].data(), stride, s);
     if (rc == kElNoRoom && n_done == 0) return rc;
     if (rc == kElNoRoom) return cuda_fail("element run kernel launch", cudaErrorCooperativeLaunchTooLarge);
     if (rc != HEOM_OK) return rc;

@@ -103,6 +103,7 @@ struct ElSmem {
   uint32_t *rng;     // [cnt][n] records of (ADO, state): begin | end << 16, relative to the chunk's first
   int2 *rest;        // [cnt][pitch] the tiles' third limbs, Re and Im (fixed point)
   int2 *hrest;       // [n][n] those of H and Im H
+  double2 *hd;       // [n][n] H and Im H in FP64, for the FMA chain
   int *key;          // [cnt][2] largest |Re|, |Im| of an ADO's tile: FP64 high word (fixed point)
   int *hkey;         // the same of H
   uint16_t *pair;    // element p of an ADO: i << 8 | j
@@ -116,7 +117,7 @@ __host__ __device__ inline size_t el_smem_bytes(int n, int cnt, int pitch, int p
   b = (b + 15) & ~(size_t)15;
   b += (size_t)cnt * pitch * 2 * real_bytes;
   b = (b + 15) & ~(size_t)15;
-  if (real_bytes == 8) b += (((size_t)cnt * pitch + (size_t)n * n) * 8 + 15) & ~(size_t)15;  // third limbs
+  if (real_bytes == 8) b += ((((size_t)cnt * pitch + (size_t)n * n) * 8 + 15) & ~(size_t)15) + (size_t)n * n * 16;  // third limbs, hd
   b += (size_t)cnt * n * 4 + (size_t)cnt * 8 + 16 + (size_t)pairs * 2;
   return (b + 15) & ~(size_t)15;
 }
@@ -141,6 +142,8 @@ __device__ __forceinline__ ElSmem<CT> el_carve(unsigned char *p, int n, int cnt,
   s.rest = reinterpret_cast<int2 *>(a);
   s.hrest = s.rest + (size_t)cnt * pitch;
   if (sizeof(CT) == 8) a = (a + ((size_t)cnt * pitch + (size_t)n * n) * 8 + 15) & ~(uintptr_t)15;
+  s.hd = reinterpret_cast<double2 *>(a);
+  if (sizeof(CT) == 8) a += (size_t)n * n * 16;
   s.rng = reinterpret_cast<uint32_t *>(a);
   s.key = reinterpret_cast<int *>(s.rng + cnt * n);  // then the key of H
   s.pair = reinterpret_cast<uint16_t *>(s.key + 2 * cnt + 4);
@@ -196,8 +199,9 @@ __device__ __forceinline__ void el_fix_consts(const ElSmem<double> &s, int n) {
   const int ex = fx_exp(*s.hkey);
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     int2 rest = make_int2(0, 0);
-    reinterpret_cast<int2 *>(s.H)[e] = fx_split3(s.H[e], ex, rest.x);
-    if (CPLX) reinterpret_cast<int2 *>(s.Hi)[e] = fx_split3(s.Hi[e], ex, rest.y);
+    s.hd[e] = make_double2(s.H[e], CPLX ? s.Hi[e] : 0.0);
+    reinterpret_cast<int2 *>(s.H)[e] = fx_split(s.H[e], ex, rest.x);
+    if (CPLX) reinterpret_cast<int2 *>(s.Hi)[e] = fx_split(s.Hi[e], ex, rest.y);
     s.hrest[e] = rest;
   }
 }
@@ -233,18 +237,18 @@ __device__ __forceinline__ void el_fix_tiles(const ElSmem<double> &s, int n, int
     const int la = e / pitch;
     const double2 z = s.tile[e];
     int2 rest;
-    const int2 a = fx_split3(z.x, fx_exp(s.key[2 * la]), rest.x), b = fx_split3(z.y, fx_exp(s.key[2 * la + 1]), rest.y);
+    const int2 a = fx_split(z.x, fx_exp(s.key[2 * la]), rest.x), b = fx_split(z.y, fx_exp(s.key[2 * la + 1]), rest.y);
     reinterpret_cast<int4 *>(s.tile)[e] = make_int4(a.x, a.y, b.x, b.y);
     s.rest[e] = rest;
   }
   __syncthreads();
 }
 
-// C = H z - z H of element (i, j) of ADO u from the limbs, or by FMAs where fixed point does not fit.
+// C = H z - z H of element (i, j) of ADO u from the limbs; bits 0 and 1 of the result: Re C, Im C is weak (fx_weak).
 template <bool CPLX>
-__device__ __forceinline__ void el_fix_comm(const ElSmem<double> &s, int n, int la, int pitch, int i, int j, double &cr,
-                                            double &ci) {
-  FxLong r, m;
+__device__ __forceinline__ int el_fix_comm(const ElSmem<double> &s, int n, int la, int pitch, int i, int j, double &cr,
+                                           double &ci) {
+  FxSum r, m;
   const int4 *z = reinterpret_cast<const int4 *>(s.tile) + la * pitch;
   const int4 *zi = z + i * n, *zj = z + j;
   const int2 *wi = s.rest + la * pitch + i * n, *wj = s.rest + la * pitch + j;
@@ -269,44 +273,31 @@ __device__ __forceinline__ void el_fix_comm(const ElSmem<double> &s, int n, int 
       m.add(-g2.x, -g2.y, -r2.y, b.x, b.y, br.x);
     }
   }
-  // a zero tile part (or H): any exponent in range
-  const int hk = *s.hkey, eh = fx_exp(hk) - 2042 - 3 * kFxLong, kx = s.key[2 * la], ky = s.key[2 * la + 1];
-  cr = r.value(hk && kx ? eh + fx_exp(kx) : 0);
-  ci = m.value(hk && ky ? eh + fx_exp(ky) : 0);
+  return fx_finish(r, m, *s.hkey, s.key[2 * la], s.key[2 * la + 1], cr, ci);
 }
 
-// The same by FP64 FMAs, from global memory.
+// C = H z - z H of element (i, j) by FP64 FMAs; h: H and Im H in shared memory, z: the ADO's tile in global memory.  (With
+// H read from global memory and H(t) put together in every term the first steps of a pulse, where many sums are
+// weak, took a third longer.)
 template <bool CPLX>
-__device__ __noinline__ void el_fma_comm(const ElConsts &kc, const double2 *z, int n, int i, int j, double gr, double gi,
-                                         double &cr, double &ci) {
+__device__ __noinline__ double2 el_fma_comm(const double2 *h, const double2 *z, int n, int i, int j) {
   double ar = 0, ai = 0, br = 0, bi = 0;
-  auto h_of = [&](int p, int q, double &re, double &im) {
-    re = kc.H[p * n + q];
-    im = kc.Hi[p * n + q];
-    if (kc.mup) {
-      const double a = kc.mup[p * n + q], b = kc.mup[q * n + p];
-      re = re - gr * (a + b);
-      im = im - gi * a + gi * b;
-    }
-  };
+#pragma unroll 4
   for (int k = 0; k < n; ++k) {
     const double2 a = __ldcg(z + k * n + j), b = __ldcg(z + i * n + k);
-    double h1, g1, h2, g2;
-    h_of(i, k, h1, g1);
-    h_of(k, j, h2, g2);
-    ar = fma(h1, a.x, ar);
-    ai = fma(h1, a.y, ai);
-    br = fma(b.x, h2, br);
-    bi = fma(b.y, h2, bi);
+    const double2 h1 = h[i * n + k], h2 = h[k * n + j];
+    ar = fma(h1.x, a.x, ar);
+    ai = fma(h1.x, a.y, ai);
+    br = fma(b.x, h2.x, br);
+    bi = fma(b.y, h2.x, bi);
     if (CPLX) {
-      ar = fma(-g1, a.y, ar);
-      ai = fma(g1, a.x, ai);
-      br = fma(-b.y, g2, br);
-      bi = fma(b.x, g2, bi);
+      ar = fma(-h1.y, a.y, ar);
+      ai = fma(h1.y, a.x, ai);
+      br = fma(-b.y, h2.y, br);
+      bi = fma(b.x, h2.y, bi);
     }
   }
-  cr = ar - br;
-  ci = ai - bi;
+  return make_double2(ar - br, ai - bi);
 }
 
 // Link ranges of the chunk [u0, u0 + cnt), cnt <= 32, records [lo, hi) at recs (already offset): a record
@@ -330,8 +321,6 @@ __device__ __forceinline__ void el_ranges(const ElSmem<CT> &s, const StageCommon
 struct ElStage {
   StateView zin, y, out, y2, out2;  // y / y2: base (none: null); out2: second output (null: none)
   double c1, c2;
-  ElConsts k;
-  double gr, gi;
 };
 
 __device__ __forceinline__ bool el_set(const StateView &v) { return v.head != nullptr || v.body != nullptr; }
@@ -419,12 +408,16 @@ __device__ __forceinline__ void el_unit(const ElSmem<CT> &s, const StageCommon &
     const CT gs = (CT)__ldg(c.gsum + u0 + la);
     CT rr, ri;
     if constexpr (FORM != kElRowOrder) {
-      CT cr, ci;  // C = H z - z H
+      CT cr = 0, ci = 0;  // C = H z - z H
       if constexpr (FORM == kElFixed) {
-        if (fx_ok(*s.hkey, s.key[2 * la]) && fx_ok(*s.hkey, s.key[2 * la + 1])) {
-          el_fix_comm<CPLX>(s, n, la, pitch, i, j, cr, ci);
-        } else {
-          el_fma_comm<CPLX>(g.k, el_own<CT, BT, OWN_HEAD>(g.zin, c, u0 + la), n, i, j, g.gr, g.gi, cr, ci);
+        int chain = 3;
+        if (fx_ok(*s.hkey, s.key[2 * la]) && fx_ok(*s.hkey, s.key[2 * la + 1]))
+          chain = el_fix_comm<CPLX>(s, n, la, pitch, i, j, cr, ci);
+        if (herm && i == j) chain &= 2;  // Re C = 0 there and is not used
+        if (chain) {
+          const double2 x = el_fma_comm<CPLX>(s.hd, el_own<CT, BT, OWN_HEAD>(g.zin, c, u0 + la), n, i, j);
+          if (chain & 1) cr = x.x;
+          if (chain & 2) ci = x.y;
         }
       } else {
         CT ar = 0, ai = 0, br = 0, bi = 0;
@@ -704,14 +697,14 @@ __global__ void __launch_bounds__(kElThreads, 2) el_stage_kernel(const __grid_co
     el_fix_consts<CPLX>(s, c.n);
     __syncthreads();
   }
-  const ElStage g{c.zin, c.y, c.out, a.y2, a.out2, a.c1, a.c2, k, a.gr, a.gi};
+  const ElStage g{c.zin, c.y, c.out, a.y2, a.out2, a.c1, a.c2};
   bool built = false;
   el_units<CT, BT, FORM, CPLX, true>(s, c, g, ElPlan{a.apu, a.splits}, blockIdx.x, gridDim.x, built);
 }
 
 // The FP64 heads of many runs of equal n_states and equal form in one launch: every CTA takes the units of its run's
 // head that fall to it.
-template <bool LEAN>
+template <bool LEAN, bool FIXED>
 __global__ void __launch_bounds__(kElThreads, 2) head_list_kernel(const __grid_constant__ HeadList L) {
   extern __shared__ __align__(16) unsigned char el_sm[];
   __shared__ StageCommon c;
@@ -735,9 +728,9 @@ __global__ void __launch_bounds__(kElThreads, 2) head_list_kernel(const __grid_c
   const ElConsts k = d->k;
   const int rank = blockIdx.x - L.cta0[lo], ncta = L.cta0[lo + 1] - L.cta0[lo];
   if constexpr (LEAN) {
-    const LeanSmem s = lean_carve(el_sm, L.n, L.apu, 0, lean_fixed(L.n, c.u_split));
-    lean_consts(s, k, L.n);
-    lean_chunks<float>(s, lean_pair(L.n), c, L.ch, k, rank, ncta);
+    const LeanSmem s = lean_carve(el_sm, L.n, L.apu, 0);
+    lean_consts<FIXED>(s, k, L.n);
+    lean_chunks<float, FIXED>(s, lean_pair(L.n), c, L.ch, k, rank, ncta);
   } else {
     const ElSmem<double> s = el_carve<double>(el_sm, L.n, L.apu, c.E, el_pairs(L.n, L.herm), true);
     el_consts<double>(s, k, L.n, L.herm, true, 0.0, 0.0);
@@ -745,7 +738,7 @@ __global__ void __launch_bounds__(kElThreads, 2) head_list_kernel(const __grid_c
     el_fix_consts<false>(s, L.n);
     __syncthreads();
     const StateView none{nullptr, nullptr};
-    const ElStage g{c.zin, c.y, c.out, none, none, L.ch, 0.0, k, 0.0, 0.0};
+    const ElStage g{c.zin, c.y, c.out, none, none, L.ch, 0.0};
     bool built = false;
     el_units<double, float, kElFixed, false, false>(s, c, g, ElPlan{L.apu, L.splits}, rank, ncta, built);
   }
@@ -783,19 +776,21 @@ __device__ __forceinline__ bool el_barrier(unsigned *bar, unsigned target, int *
 }
 
 // The FP64 head of a mixed run, out of line (its shared memory at the start of the dynamic part).
-__device__ __noinline__ void lean_chunks_of_head(int n, int a, bool fixed, const StageCommon &cr, double ch, const ElConsts &kc,
+template <bool FIXED>
+__device__ __noinline__ void lean_chunks_of_head(int n, int a, const StageCommon &cr, double ch, const ElConsts &kc,
                                                  int first, int stride) {
   extern __shared__ __align__(16) unsigned char el_sm[];
   const StageCommon c = cr;
-  lean_chunks<float>(lean_carve(el_sm, n, a, 0, fixed), lean_pair(n), c, ch, kc, first, stride);
+  lean_chunks<float, FIXED>(lean_carve(el_sm, n, a, 0), lean_pair(n), c, ch, kc, first, stride);
 }
 
-// The kinds of el_run_kernel, one per set of code that its CTAs hold: FP64 runs that the pair kernels cover, with
+// The kinds of el_run_kernel, one per set of code that its CTAs hold (FIXED: with the pair kernels' commutator in fixed
+// point; as a branch it cost the runs without it 10 % in registers): FP64 runs that the pair kernels cover, with
 // every ADO kept by a CTA or in chunks; mixed runs whose head they cover (with the row form for the body); and
 // all others.
 constexpr int kRunKept = 0, kRunMixed = 1, kRunOther = 2, kRunChunks = 3;
 
-template <int KIND>
+template <int KIND, bool FIXED>
 __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThreads, 2) el_run_kernel(const __grid_constant__ ElList L) {
   extern __shared__ __align__(16) unsigned char el_sm[];
   __shared__ ElRunDesc d;
@@ -843,12 +838,11 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
   const bool rows = KIND == kRunMixed || d.c.herm;
   if (do64) {
     if constexpr (KIND != kRunOther) {
-      const int64_t part = cs[0][0].u_end;
-      sl = lean_carve(top, n, en.apu64, KIND == kRunKept ? kLeanRunThreads : 0, lean_fixed(n, part));
+      sl = lean_carve(top, n, en.apu64, KIND == kRunKept ? kLeanRunThreads : 0);
       top = sl.end;
-      lean_consts(sl, d.k, n);
+      lean_consts<FIXED>(sl, d.k, n);
       lp = lean_pair(n);
-      if constexpr (KIND == kRunKept) lean_begin<double>(ls, sl, lp, cs[0][0], rank, n64);
+      if constexpr (KIND == kRunKept) lean_begin<double, FIXED>(ls, sl, lp, cs[0][0], rank, n64);
     } else {
       const int P = el_pairs(n, d.c.herm);
       s64 = el_carve<double>(top, n, en.apu64, d.fp64 ? d.c.Ep : d.c.E, P, true);
@@ -889,17 +883,16 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
         g.out = cs[0][q].out;
         g.y2 = g.out2 = StateView{nullptr, nullptr};
         g.c1 = ch;
-        g.c2 = g.gr = g.gi = 0;
-        g.k = d.k;
+        g.c2 = 0;
       }
       if (do64) {
         const StageCommon &c = cs[0][q];
         if constexpr (KIND == kRunKept) {
-          lean_step<double>(ls, sl, lp, c, ch, d.k, q == 0);
+          lean_step<double, FIXED>(ls, sl, lp, c, ch, d.k, q == 0);
         } else if constexpr (KIND == kRunChunks) {
-          lean_chunks<double>(sl, lp, c, ch, d.k, rank, n64);
+          lean_chunks<double, FIXED>(sl, lp, c, ch, d.k, rank, n64);
         } else if constexpr (KIND == kRunMixed) {
-          lean_chunks_of_head(n, en.apu64, sl.fixed, c, ch, d.k, rank, n64);
+          lean_chunks_of_head<FIXED>(n, en.apu64, c, ch, d.k, rank, n64);
         } else {
           const ElPlan pl{en.apu64, en.split64};
           if (d.fp64) {

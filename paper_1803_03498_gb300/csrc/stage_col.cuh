@@ -13,17 +13,18 @@
 //
 // Bound and form: GB300 issues one FP64 instruction per 64 clocks and SM partition (18.7 clocks per SM measured), two
 // 32 x 32 + 64 bit integer multiply-adds per clock and SM.  The commutator, 2 N^3 multiply-adds per ADO, therefore runs
-// in exact integers (fixed_point.cuh: two limbs of 29 bits, one rounding at the end of a sum), and the FP64 pipe keeps
+// in integers (fixed_point.cuh: three limbs of 28 bits, one rounding at the end of a sum), and the FP64 pipe keeps
 // what is cheaper there than in integers: the sums' conversion (2 additions), the decay, the links (2 per
 // record and lane), R and the RK4 combination (4 per pair of elements).  A lane owns one column of one part: lane (a, p, j)
 // computes column j of Q_re (p = 0, from H Im s) or of Q_im (p = 1, from -H Re s) of ADO a -- 2N columns
 // per ADO -- so the scale of its operands is its own column's largest element, without a word to other lanes, and
-// the limbs of H enter every multiply-add as kernel-parameter (constant-bank) operands.  A warp takes chunks of G
+// the limbs of H come from shared memory, one 16-byte broadcast each (as 16-byte constant loads: 187 ms against 177 for
+// four steps at the LHCII size).  A warp takes chunks of G
 // consecutive ADOs, G chosen so that 2 N G is a multiple of 32, and covers their 2 N G columns in P = 2 N G / 32
 // passes with every lane busy (N = 14: 8 ADOs in 7 passes).  Per pass a lane
 //   - loads column j of its ADO's zin tile from global memory (the 2N lanes of an ADO read whole rows:
 //     coalesced) and splits the part it multiplies into limbs;
-//   - forms the N entries of its column of H (Im s) or -H (Re s), each a sum of 4 N integer products, plus
+//   - forms the N entries of its column of H (Im s) or -H (Re s), each a sum of 6 N integer products, plus
 //     coef * (own part);
 //   - writes the column in FP64 into its ADO's slot of a per-warp ring of Q tiles in shared memory.
 // An ADO whose last column was computed in this pass is finalised by the warp: the
@@ -31,7 +32,8 @@
 // is added to row s of Q, records in order; then the lanes take the pairs i <= j: R_ij = Q_ij + conj(Q_ji),
 // out = y + ch R, written to (i, j) and, conjugated, to (j, i).  Warps are independent (only __syncwarp).  Every output
 // element sums the same terms in the same order under every launch schedule.
-// A column with Inf, NaN or exponents near the ends of the range takes FP64 FMAs instead.
+// A column with Inf, NaN or exponents near the ends of the range takes FP64 FMAs instead, and so does a row of it whose sum
+// is weak beside the column (fx_weak).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -141,26 +143,30 @@ __device__ __forceinline__ void col_links(const LinkRec<double> *rec, int nr, co
   if (cur >= 0) qp[cur * N + j] = acc;
 }
 
-constexpr int kColBits = 29;  // sums of N <= 16 products of 2^56 and twice as many cross products fit 63 bits
-
 struct ColArgs {
   StageCommon c;
   double ch;
   int ex;                                // |H| < 2^(ex - 1022)
   double term[kMaxStates];               // terminator Delta per state
   double H[kMaxStates * kMaxStates];     // Re H - h0 I, rad/fs (columns out of range)
-  int2 Hx[kMaxStates * kMaxStates];      // its limbs
+  int4 Hx[kMaxStates * kMaxStates];      // its limbs
 };
 
-// Column j of part p of -i H s + coef s by FP64 FMAs, into q[i * N + j].
+// Row i of column zt[0], zt[N], ... of H Im s (p = 0) or -H Re s (p = 1) by FP64 FMAs.
+template <int N>
+__device__ __noinline__ double col_fma_row(const ColArgs &a, const double2 *zt, int p, int i) {
+  double acc = 0;
+  for (int k = 0; k < N; ++k) {
+    const double2 z = zt[k * N];
+    acc = fma(a.H[i * kMaxStates + k], p ? -z.x : z.y, acc);
+  }
+  return acc;
+}
+// Column j of part p of -i H s + coef s the same way, into q[i * N + j].
 template <int N>
 __device__ __noinline__ void col_fma(const ColArgs &a, const double2 *zt, int p, int j, double g, double *q) {
   for (int i = 0; i < N; ++i) {
-    double acc = 0;
-    for (int k = 0; k < N; ++k) {
-      const double2 z = zt[k * N];
-      acc = fma(a.H[i * kMaxStates + k], p ? -z.x : z.y, acc);
-    }
+    const double acc = col_fma_row<N>(a, zt, p, i);
     const double2 z = zt[i * N];
     q[i * N + j] = fma(i == j ? -0.5 * g : fma(-0.5, g, -a.term[i]), p ? z.y : z.x, acc);
   }
@@ -172,6 +178,9 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
   using W = ColSmem<N>;
   constexpr int C = S::C, G = S::G, P = S::P, E = S::E, RB = S::RB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int4 Hs[N * N];  // the limbs of H
+  for (int e = threadIdx.x; e < N * N; e += blockDim.x) Hs[e] = a.Hx[(e / N) * kMaxStates + e % N];
+  __syncthreads();
   const StageCommon &c = a.c;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char *wb = smem_raw + warp * W::total;
@@ -251,24 +260,35 @@ __global__ void __launch_bounds__(ColShape<N>::WARPS * 32, 4) stage_col_kernel(c
         if (fx_ok(a.ex << 20, key)) {
           const int ex = fx_exp(key);
           int2 src[N];
+          int rest[N];
 #pragma unroll
-          for (int k = 0; k < N; ++k) src[k] = fx_split(p ? col_neg(zc[k]) : zc[k], ex, kColBits);
+          for (int k = 0; k < N; ++k) src[k] = fx_split(p ? col_neg(zc[k]) : zc[k], ex, rest[k]);
           const double *cf = coef + ad * N;
           const double gd = gh[ad];
-          const int e2 = key ? a.ex - 2042 - 2 * kColBits + ex : 0;  // a zero column: any scale in range
+          const int e2 = key ? fx_unit(a.ex << 20, key) : 0;  // a zero column: any scale in range
+          unsigned weak = 0;  // rows to be taken from the FMA chain: after the loop, whose rows then overlap
           const double *zo = reinterpret_cast<const double *>(zin + (int64_t)(u0 + ad) * Ep + j) + p;  // own part
-          // Rows in a loop, two at a time: unrolled over all of them (2700 instructions) the code outgrew the instruction
-          // cache and the kernel took 20 ms at the LHCII size; one at a time 8.8 ms, two 8.4 (5 CTAs per SM: 9.4)
-#pragma unroll 2
+          // Rows in a loop, one at a time: unrolled over all of them the code outgrew the instruction cache and the kernel
+          // took more than twice as long (two limbs: 20 ms per launch against 8.4); two at a time 182 ms for four steps at the
+          // LHCII size, one 177 (3 CTAs per SM with 168 registers: 188)
+#pragma unroll 1
           for (int i = 0; i < N; ++i) {
             const double own = zo[2 * i * N], ci = i == j ? gd : cf[i];
             FxSum r;
 #pragma unroll
             for (int k = 0; k < N; ++k) {
-              const int2 hx = a.Hx[i * kMaxStates + k];
-              r.add(hx.x, hx.y, src[k].x, src[k].y);
+              const int4 hx = Hs[i * N + k];
+              r.add(hx.x, hx.y, hx.z, src[k].x, src[k].y, rest[k]);
             }
-            qs[i * N + j] = fma(ci, own, fx_double_add(r.total(kColBits), e2));
+            unsigned f;
+            const long long w = r.whole(f);
+            weak |= (unsigned)fx_weak(w) << i;
+            qs[i * N + j] = fma(ci, own, fx_double_add(w, f, e2));
+          }
+          if (weak && key) {
+            for (int i = 0; i < N; ++i)
+              if (weak >> i & 1)
+                qs[i * N + j] = fma(i == j ? gd : cf[i], zo[2 * i * N], col_fma_row<N>(a, zin + (int64_t)(u0 + ad) * Ep + j, p, i));
           }
         } else {
           col_fma<N>(a, zin + (int64_t)(u0 + ad) * Ep + j, p, j, c.gsum[u0 + ad], qs);
@@ -335,17 +355,18 @@ int launch_col(const StageCommon &c, double ch, const double *term, const double
   for (int i = 0; i < kMaxStates; ++i) a.term[i] = (i < c.n) ? term[i] : 0.0;
   for (int i = 0; i < kMaxStates * kMaxStates; ++i) {
     a.H[i] = 0.0;
-    a.Hx[i] = make_int2(0, 0);
+    a.Hx[i] = make_int4(0, 0, 0, 0);
   }
   for (int i = 0; i < c.n; ++i)
     for (int j = 0; j < c.n; ++j) {
       const double h = H[i * c.n + j];
       a.H[i * kMaxStates + j] = h;
       if (a.ex == 2047) continue;
-      // as fx_split: |h| < 2^(ex - 1022), rounded to 2 kColBits - 1 bits
-      const long long v = std::llrint(std::ldexp(h, 2 * kColBits - 1 - (a.ex - 1022)));
-      const long long lo = ((v + (1ll << (kColBits - 1))) & ((1ll << kColBits) - 1)) - (1ll << (kColBits - 1));
-      a.Hx[i * kMaxStates + j] = make_int2((int)((v - lo) >> kColBits), (int)lo);
+      // as fx_split: |h| < 2^(ex - 1022); the last limb rounded
+      const double x = std::ldexp(h, 2 * kFxBits - 1 - (a.ex - 1022));
+      const long long v = std::llrint(x);
+      const long long lo = ((v + (1ll << (kFxBits - 1))) & ((1ll << kFxBits) - 1)) - (1ll << (kFxBits - 1));
+      a.Hx[i * kMaxStates + j] = make_int4((int)((v - lo) >> kFxBits), (int)lo, (int)std::llrint(std::ldexp(x - (double)v, kFxBits)), 0);
     }
   constexpr int WARPS = ColShape<N>::WARPS;
   const size_t smem = (size_t)WARPS * ColSmem<N>::total;
