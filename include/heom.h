@@ -179,7 +179,7 @@ int heom_run_destroy(heom_run *r);
  * (four evaluations of the right-hand side of Eq. HEOM per step).  Every obs_stride steps (0 =
  * never) one observable record of sigma_0 is appended after the step.  Enqueued on the run's
  * stream; does not block.  Small hierarchies advance many steps per (cooperative) launch, whose CTAs meet
- * at a barrier after every stage (bounded: HEOM_E_TIMEOUT from heom_observables if it gave up); with kernel
+ * at a barrier after every stage (bounded: HEOM_E_TIMEOUT from the calls that return results if it gave up); with kernel
  * timing on, under stream capture, or in a context with too few SMs for the launch, every stage is a launch
  * of its own, with the same results.  Errors: HEOM_E_ARG (dt_fs <= 0, n_steps < 0, dt_fs times the fastest
  * decay rate D * max gamma above 2.5, where RK4 is no longer stable), HEOM_E_NOMEM (the records
@@ -230,12 +230,13 @@ int heom_record_len(const heom_run *r);
 int heom_observables(heom_run *r, double *out, int64_t cap_records, int64_t *written);
 
 /* Synchronises; copies the reduced density matrix rho = sigma_0 (the root ADO, section "HEOM
- * formalism"; FP64 in every precision) into caller host arrays of n_states^2 doubles, row-major. */
+ * formalism"; FP64 in every precision) into caller host arrays of n_states^2 doubles, row-major.
+ * HEOM_E_TIMEOUT and HEOM_E_BOUNDS as heom_observables. */
 int heom_get_sigma0(heom_run *r, double *re, double *im);
 
 /* Synchronises; copies ADOs [u0, u0 + count) of the current state into / out of caller host
  * arrays [count][N][N] (FP32-stored ADOs are rounded on the way in).  HEOM_E_ARG if the range is
- * outside [0, n_ado). */
+ * outside [0, n_ado); heom_get_ados: HEOM_E_TIMEOUT and HEOM_E_BOUNDS as heom_observables. */
 int heom_get_ados(heom_run *r, int64_t u0, int64_t count, double *re, double *im);
 int heom_set_ados(heom_run *r, int64_t u0, int64_t count, const double *re, const double *im);
 
@@ -243,7 +244,7 @@ int heom_set_ados(heom_run *r, int64_t u0, int64_t count, const double *re, cons
  * heom_rhs_eval -- evaluate the right-hand side of Eq. HEOM once on the current state with the
  * same kernels heom_propagate uses, and copy ADOs [u0, u0 + count) of d sigma / dt into caller
  * host arrays [count][N][N].  The state is not changed (the result goes through a scratch copy of
- * the workspace).  Synchronises.
+ * the workspace).  Synchronises.  HEOM_E_TIMEOUT and HEOM_E_BOUNDS as heom_observables.
  */
 int heom_rhs_eval(heom_run *r, int64_t u0, int64_t count, double *re, double *im);
 

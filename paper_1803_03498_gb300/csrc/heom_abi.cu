@@ -869,8 +869,8 @@ extern "C" int heom_set_ados(heom_run *r, int64_t u0, int64_t count, const doubl
 
 extern "C" int heom_get_ados(heom_run *r, int64_t u0, int64_t count, double *re, double *im) {
   if (!r) { set_error("heom_get_ados: NULL run"); return HEOM_E_ARG; }
-  cudaError_t e = cudaStreamSynchronize(r->stream);
-  if (e != cudaSuccess) return cuda_fail("heom_get_ados: stream", e);
+  const int rc = device_status(r, "heom_get_ados", nullptr);
+  if (rc) return rc;
   return io_range(r, r->y, u0, count, re, im, false);
 }
 

@@ -16,8 +16,8 @@ constexpr int kGenMaxStates = 32;  // states of general runs (element kernels on
 void set_error(const std::string &msg);
 
 // Device error word of a run (StageCommon::err): bit 0 -- a bounded device-side wait gave up (the
-// tensor-core kernel's, or the barrier of a launch of whole steps); bit 1 -- a bounds check of the debug build failed.  heom_observables reports
-// them as HEOM_E_TIMEOUT and HEOM_E_BOUNDS.
+// tensor-core kernel's, or the barrier of a launch of whole steps); bit 1 -- a bounds check of the debug build failed.  Every call that returns
+// results of the run reports them as HEOM_E_TIMEOUT and HEOM_E_BOUNDS.
 constexpr int kErrTimeout = 1;
 constexpr int kErrBounds = 2;
 

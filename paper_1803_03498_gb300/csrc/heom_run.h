@@ -106,6 +106,7 @@ namespace heom {
 // count check (graph capture: heom_batch_launch checks the counts per replay); the kernel keeps
 // the run's real max_records as its bound either way.
 int enqueue_record(heom_run *r, bool host_check = true);
+int device_status(heom_run *r, const char *who, int64_t *records);
 int io_range(heom_run *r, StateView state, int64_t u0, int64_t count, double *re, double *im, bool to_device);
 
 // the RK4 driver (propagate.cu)

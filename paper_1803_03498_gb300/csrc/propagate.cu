@@ -292,26 +292,35 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
   return HEOM_OK;
 }
 
-extern "C" int heom_observables(heom_run *r, double *out, int64_t cap_records, int64_t *written) {
-  if (!r || !out || cap_records < 0) { set_error("heom_observables: bad arguments"); return HEOM_E_ARG; }
-  cudaError_t e = cudaStreamSynchronize(r->stream);
-  if (e != cudaSuccess) return cuda_fail("heom_observables: stream", e);
+// Waits for the run's stream and reads its device error word (and the number of records): every call that hands results
+// to the caller asks for it first.
+int heom::device_status(heom_run *r, const char *who, int64_t *records) {
   int64_t cnt_err[2] = {0, 0};
-  e = cudaMemcpy(cnt_err, r->rec_count, sizeof(cnt_err), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail("heom_observables: counter", e);
+  cudaError_t e = cudaMemcpyAsync(cnt_err, r->rec_count, sizeof(cnt_err), cudaMemcpyDeviceToHost, r->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
+  if (e != cudaSuccess) return cuda_fail(who, e);
+  if (records) *records = cnt_err[0];
   int err_flag = 0;
   std::memcpy(&err_flag, &cnt_err[1], sizeof(int));
   if (err_flag & kErrBounds) {
-    set_error("heom_observables: a bounds check of the debug build failed (a link record names an ADO, state or "
+    set_error(std::string(who) + ": a bounds check of the debug build failed (a link record names an ADO, state or "
               "record range outside the run; its results are invalid)");
     return HEOM_E_BOUNDS;
   }
   if (err_flag) {
-    set_error("heom_observables: a bounded device-side wait gave up (the tensor-core kernel's, or the barrier of a launch of whole "
-              "steps; the run's results are invalid)");
+    set_error(std::string(who) + ": a bounded device-side wait gave up (the tensor-core kernel's, or the barrier of a launch "
+              "of whole steps; the run's results are invalid)");
     return HEOM_E_TIMEOUT;
   }
-  int64_t cnt = cnt_err[0];
+  return HEOM_OK;
+}
+
+extern "C" int heom_observables(heom_run *r, double *out, int64_t cap_records, int64_t *written) {
+  if (!r || !out || cap_records < 0) { set_error("heom_observables: bad arguments"); return HEOM_E_ARG; }
+  int64_t cnt = 0;
+  const int rc = device_status(r, "heom_observables", &cnt);
+  if (rc) return rc;
+  cudaError_t e = cudaSuccess;
   cnt = std::min(cnt, cap_records);
   const int rl = r->n + 5;
   if (cnt > 0) {
@@ -334,7 +343,6 @@ extern "C" int heom_rhs_eval(heom_run *r, int64_t u0, int64_t count, double *re,
   if (r->has_field) field_g(r, r->t_fs);  // L at the current time
   int rc = run_stage(r, r->y, none, r->zA, 1.0);
   if (rc) return rc;
-  cudaError_t e = cudaStreamSynchronize(r->stream);
-  if (e != cudaSuccess) return cuda_fail("heom_rhs_eval: stream", e);
+  if ((rc = device_status(r, "heom_rhs_eval", nullptr))) return rc;
   return io_range(r, r->zA, u0, count, re, im, false);
 }
