@@ -165,7 +165,8 @@ __device__ __forceinline__ void col_run_part(const ColRunArgs &a, unsigned char 
 
 __global__ void __launch_bounds__(kColThreads, 2) col_run_kernel(const __grid_constant__ ColRunArgs a) {
   extern __shared__ __align__(16) unsigned char el_sm[];
-  if (*(volatile int *)a.d.c.err & kErrTimeout) return;  // an earlier launch of this run gave up
+  // an earlier launch of this run gave up: the whole CTA leaves, whatever each of its threads reads
+  if (__syncthreads_or(*(volatile int *)a.d.c.err & kErrTimeout)) return;
   const int rank = blockIdx.x, ncta = gridDim.x, n64 = a.d.fp64 ? a.d.c.n_ado : a.d.c.u_split;
   if (rank < a.hcta) {
     const int first = rank * a.apu64, cnt = max(0, min(a.apu64, n64 - first));

@@ -809,7 +809,8 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
   }
   __syncthreads();
   const int rank = blockIdx.x - en.cta0, ncta = (lo + 1 < L.nruns ? L.e[lo + 1].cta0 : (int)gridDim.x) - en.cta0;
-  if (*(volatile int *)d.c.err & kErrTimeout) return;  // an earlier launch of this run gave up
+  // an earlier launch of this run gave up: the whole CTA leaves, whatever each of its threads reads
+  if (__syncthreads_or(*(volatile int *)d.c.err & kErrTimeout)) return;
   // part 0: FP64 (every ADO of an FP64 run, the head of a mixed one); part 1: the FP32 body
   if (threadIdx.x < 8) {
     const int part = threadIdx.x >> 2, q = threadIdx.x & 3;
