@@ -231,6 +231,11 @@ struct ElEntry {
   int steps;
   int stride, first_rec;     // a record every stride steps, the first after first_rec steps (0: none)
 };
+// el_run_kernel for a mixed run of n states with a Hermitian state (nullptr: not compiled in the unit)
+const void *mixed_run_kernel_a(int n);
+const void *mixed_run_kernel_b(int n);
+const void *mixed_run_kernel_c(int n);
+const void *mixed_run_kernel_d(int n);
 constexpr int kElMaxRuns = 256;  // runs per launch (kernel parameters: about 10 KB)
 struct ElList {
   ElEntry e[kElMaxRuns];

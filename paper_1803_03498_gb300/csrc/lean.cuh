@@ -154,7 +154,7 @@ __device__ __forceinline__ void lean_limbs(const LeanSmem &s, const LeanPair &p,
 }
 
 // C = H z - z H of element (i, j) by FP64 FMAs, H and the ADO's tile z in global memory.
-__device__ __noinline__ double2 lean_fma_comm(const double *H, const double2 *z, int n, int i, int j) {
+static __device__ __noinline__ double2 lean_fma_comm(const double *H, const double2 *z, int n, int i, int j) {
   double ar = 0, ai = 0, br = 0, bi = 0;
 #pragma unroll 4
   for (int k = 0; k < n; ++k) {

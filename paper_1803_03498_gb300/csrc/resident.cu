@@ -330,15 +330,43 @@ static int kept_ctas(const heom_run *r) {
   return (int)((r->n_ado + a - 1) / a);
 }
 
-template <int KIND, bool FIXED>
-static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
-  static std::atomic<bool> ready{false};
-  if (!ready) {
-    const int rc = max_smem((const void *)el_run_kernel<KIND, FIXED>, "element run kernel");
-    if (rc) return HEOM_E_CUDA;
-    ready = true;
+// The forms of el_run_kernel (kind, fixed, states of the row form) and their kernels.
+constexpr int kFormOther = 4, kFormMixed = 8, kForms = kFormMixed + kMaxStates + 1;  // 0..3: kept, chunks; 8 + n: mixed
+static int form_of(const heom_run *r, bool kept) {
+  if (r->precision != HEOM_FP64) return r->herm ? kFormMixed + r->n : kFormOther;
+  if (!run_lean(r)) return kFormOther;
+  return (kept ? 0 : 2) + (lean_fixed(r->n, r->n_ado) ? 1 : 0);
+}
+static const void *form_kernel(int form) {
+  switch (form) {
+    case 0: return (const void *)el_run_kernel<kRunKept, false, 0>;
+    case 1: return (const void *)el_run_kernel<kRunKept, true, 0>;
+    case 2: return (const void *)el_run_kernel<kRunChunks, false, 0>;
+    case 3: return (const void *)el_run_kernel<kRunChunks, true, 0>;
+    case kFormOther: return (const void *)el_run_kernel<kRunOther, true, 0>;
   }
-  constexpr int threads = KIND == kRunKept ? kLeanRunThreads : kElThreads;
+  const int n = form - kFormMixed;
+  const void *k = mixed_run_kernel_a(n);
+  if (!k) k = mixed_run_kernel_b(n);
+  if (!k) k = mixed_run_kernel_c(n);
+  if (!k) k = mixed_run_kernel_d(n);
+  return k;
+}
+
+static int propagate_form(int form, heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
+  static std::atomic<bool> ready[kForms];
+  const void *kernel = form_kernel(form);
+  if (!kernel) {
+    set_error("element run kernel: n_states not compiled");
+    return HEOM_E_CUDA;
+  }
+  if (!ready[form]) {
+    const int rc = max_smem(kernel, "element run kernel");
+    if (rc) return HEOM_E_CUDA;
+    ready[form] = true;
+  }
+  const bool kept_form = form < 2;
+  const int threads = kept_form ? kLeanRunThreads : kElThreads;
   const int sm_count = runs[0]->sm_count, cap = 2 * sm_count;  // 2 CTAs per SM (launch bounds; kElSmemMax)
   int64_t most = 0;
   for (int i = 0; i < n_runs; ++i) most = std::max(most, steps[i]);
@@ -357,7 +385,7 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
         if (steps[i] > at) {
           in.push_back(i);
           total += cost64(runs[i]) + cost32(runs[i]);
-          if (KIND == kRunKept) kept += kept_ctas(runs[i]);
+          if (kept_form) kept += kept_ctas(runs[i]);
           const ElShare w = share_of(runs[i], cap);
           want += w.n64 == 1 && w.n32 <= 1 && cost64(runs[i]) + cost32(runs[i]) <= 2 * kElGrain ? 1 : w.n64 + w.n32;
         }
@@ -370,7 +398,7 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
         const double cost = cost64(r) + cost32(r);
         // everything each run can use, or its share of the CTAs by cost, one at least for each that follows
         int mine = cap;
-        if (KIND == kRunKept) {
+        if (kept_form) {
           mine = kept_ctas(r) + (int)(cost / total * (cap - kept));
         } else if (want > cap) {
           const int left = cap - cta - (int)(in.size() - q - 1);
@@ -383,8 +411,8 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
         // a kept run spreads until its CTAs have a warp for each partition of their SM (FP64 instructions of
         // one warp follow each other 64 clocks apart, whatever the other partitions do)
         const int64_t kept_h = std::min<int64_t>(r->n_ado, std::max<int64_t>(kept_ctas(r), std::min<int64_t>(mine, (r->n_ado * P + 127) / 128)));
-        const bool one = KIND == kRunKept ? kept_h == 1 : mine <= 1 || cost <= 2 * kElGrain;
-        const int h64 = KIND == kRunKept ? (int)kept_h : one ? 1 : w.n64, h32 = one ? 1 : w.n32;
+        const bool one = kept_form ? kept_h == 1 : mine <= 1 || cost <= 2 * kElGrain;
+        const int h64 = kept_form ? (int)kept_h : one ? 1 : w.n64, h32 = one ? 1 : w.n32;
         ElEntry &e = L.e[L.nruns++];
         e.d = reinterpret_cast<const ElRunDesc *>(r->desc_dev);
         e.cta0 = cta;
@@ -396,7 +424,7 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
         e.apu32 = nb > 0 ? (int)std::min<int64_t>((nb + h32 - 1) / h32, fit_ados(r->n, r->Ep, P, 4, false, room)) : 1;
         longest = std::max(longest, one ? cost : std::max(cost64(r) / h64, cost32(r) / std::max(1, h32)));
         e.row_bytes = nb > 0 && r->herm ? row_bytes(r->n) : 0;
-        const size_t m64 = run_lean(r) ? lean_smem_bytes(r->n, e.apu64, KIND == kRunKept ? threads : 0)
+        const size_t m64 = run_lean(r) ? lean_smem_bytes(r->n, e.apu64, kept_form ? threads : 0)
                                        : el_smem_bytes(r->n, e.apu64, pitch64, P, 8, true);
         const size_t m32 = nb <= 0 ? 0 : r->herm ? sizeof(RowConsts) + (size_t)e.row_bytes * (kElThreads / 32)
                                                : el_smem_bytes(r->n, e.apu32, r->Ep, P, 4, false);
@@ -416,7 +444,7 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
         }
       }
       void *args[] = {&L};
-      cudaError_t ce = cudaLaunchCooperativeKernel((const void *)el_run_kernel<KIND, FIXED>, dim3(cta), dim3(threads), args, smem, s);
+      cudaError_t ce = cudaLaunchCooperativeKernel(kernel, dim3(cta), dim3(threads), args, smem, s);
       if (ce == cudaSuccess) ce = cudaGetLastError();
       if (no_room(ce) && at == 0 && b0 == 0) return kElNoRoom;
       if (ce != cudaSuccess) return cuda_fail("element run kernel launch", ce);
@@ -436,32 +464,21 @@ static int propagate_kind(heom_run *const *runs, int n_runs, double h, const int
 // Steps [done, done + steps[i]) of every run on stream s, as few launches as possible; the runs' counters
 // (steps_done, t_fs, records_host, launches) advance.
 int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
-  // kRunKept, kRunMixed and kRunChunks without and with fixed point, then the others
-  constexpr int kForms = 7;
   std::vector<heom_run *> rs[kForms];
   std::vector<int64_t> st[kForms];
-  auto fixed = [](const heom_run *r) {
-    return r->precision == HEOM_FP64 ? lean_fixed(r->n, r->n_ado) : lean_head_fixed(r->n);
-  };
-  int need[2] = {0, 0};
+  int need[2] = {0, 0};  // CTAs that keep the runs without and with fixed point
   for (int i = 0; i < n_runs; ++i)
-    if (run_lean(runs[i]) && runs[i]->precision == HEOM_FP64) need[fixed(runs[i])] += kept_ctas(runs[i]);
+    if (run_lean(runs[i]) && runs[i]->precision == HEOM_FP64) need[form_of(runs[i], true)] += kept_ctas(runs[i]);
   for (int i = 0; i < n_runs; ++i) {
-    const bool fx = fixed(runs[i]);
-    const int form = !run_lean(runs[i])                     ? 6
-                     : runs[i]->precision != HEOM_FP64      ? 2 + fx
-                     : need[fx] <= 2 * runs[i]->sm_count ? 0 + fx
-                                                         : 4 + fx;
+    int form = form_of(runs[i], true);
+    if (form < 2 && need[form] > 2 * runs[i]->sm_count) form = form_of(runs[i], false);
     rs[form].push_back(runs[i]);
     st[form].push_back(steps[i]);
   }
-  static int (*const fns[kForms])(heom_run *const *, int, double, const int64_t *, int64_t, cudaStream_t) = {
-      propagate_kind<kRunKept, false>,  propagate_kind<kRunKept, true>,   propagate_kind<kRunMixed, false>, propagate_kind<kRunMixed, true>,
-      propagate_kind<kRunChunks, false>, propagate_kind<kRunChunks, true>, propagate_kind<kRunOther, true>};
   int n_done = 0;
   for (int form = 0; form < kForms; ++form) {
     if (rs[form].empty()) continue;
-    const int rc = fns[form](rs[form].data(), (int)rs[form].size(), h, st[form].data(), stride, s);
+    const int rc = propagate_form(form, rs[form].data(), (int)rs[form].size(), h, st[form].data(), stride, s);
     if (rc == kElNoRoom && n_done == 0) return rc;
     if (rc == kElNoRoom) return cuda_fail("element run kernel launch", cudaErrorCooperativeLaunchTooLarge);
     if (rc != HEOM_OK) return rc;

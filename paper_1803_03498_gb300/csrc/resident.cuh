@@ -574,7 +574,7 @@ struct RowConsts {
 // k_at, w_at: offsets of the RowConsts and of the warp's buffers in the dynamic shared memory (an address that the
 // compiler can see to be shared: through generic pointers the same code ran 3.5 times slower).
 template <int N>
-__device__ __noinline__ void row_body(int k_at, int w_at, const StageCommon &cr, float ch, int first, int nwarps) {
+__device__ __forceinline__ void row_body(int k_at, int w_at, const StageCommon &cr, float ch, int first, int nwarps) {
   using S = StageShape<N, float, float>;
   using W = RowSmem<N>;
   constexpr int A = S::A, EPO = S::EpBody;
@@ -676,7 +676,7 @@ __device__ __noinline__ void row_body(int k_at, int w_at, const StageCommon &cr,
 
 // f(std::integral_constant<int, N>) for N = n in LO..HI.
 template <int LO, int HI, typename F>
-__host__ __device__ __forceinline__ void row_dispatch(int n, F f) {
+inline void row_dispatch(int n, F f) {
   if (n == LO) f(std::integral_constant<int, LO>{});
   else if constexpr (LO < HI) row_dispatch<LO + 1, HI>(n, f);
 }
@@ -775,22 +775,15 @@ __device__ __forceinline__ bool el_barrier(unsigned *bar, unsigned target, int *
   return ok != 0;
 }
 
-// The FP64 head of a mixed run, out of line (its shared memory at the start of the dynamic part).
-template <bool FIXED>
-__device__ __noinline__ void lean_chunks_of_head(int n, int a, const StageCommon &cr, double ch, const ElConsts &kc,
-                                                 int first, int stride) {
-  extern __shared__ __align__(16) unsigned char el_sm[];
-  const StageCommon c = cr;
-  lean_chunks<float, FIXED>(lean_carve(el_sm, n, a, 0), lean_pair(n), c, ch, kc, first, stride);
-}
-
 // The kinds of el_run_kernel, one per set of code that its CTAs hold (FIXED: with the pair kernels' commutator in fixed
-// point; as a branch it cost the runs without it 10 % in registers): FP64 runs that the pair kernels cover, with
-// every ADO kept by a CTA or in chunks; mixed runs whose head they cover (with the row form for the body); and
-// all others.
+// point; as a branch it cost the runs without it 10 % in registers; ROWS: the states of a Hermitian FP32 body in row form, or
+// 0): FP64 runs that the pair kernels cover, with every ADO kept by a CTA or in chunks; mixed runs whose head they
+// cover; and all others.  A kernel for each number of states, with its code in line: the row form as functions called
+// from one kernel had a stack of 2.6 KB a thread to save registers in, 0.47 GB of device memory that the
+// runtime takes at the first such launch.
 constexpr int kRunKept = 0, kRunMixed = 1, kRunOther = 2, kRunChunks = 3;
 
-template <int KIND, bool FIXED>
+template <int KIND, bool FIXED, int ROWS>
 __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThreads, 2) el_run_kernel(const __grid_constant__ ElList L) {
   extern __shared__ __align__(16) unsigned char el_sm[];
   __shared__ ElRunDesc d;
@@ -836,7 +829,6 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
   ElSmem<double> s64{};
   ElSmem<float> s32{};
   int k_at = 0, w_at = 0;  // the FP32 body's constants and this warp's buffers in el_sm
-  const bool rows = KIND == kRunMixed || d.c.herm;
   if (do64) {
     if constexpr (KIND != kRunOther) {
       sl = lean_carve(top, n, en.apu64, KIND == kRunKept ? kLeanRunThreads : 0);
@@ -850,12 +842,12 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
       top = s64.end;
       el_consts<double>(s64, d.k, n, d.c.herm, true, 0.0, 0.0);
       __syncthreads();
-      if (d.c.cplx_h) el_fix_consts<true>(s64, n);
+      if (ROWS == 0 && d.c.cplx_h) el_fix_consts<true>(s64, n);
       else el_fix_consts<false>(s64, n);
     }
   }
   if (do32) {
-    if (rows) {
+    if constexpr (ROWS > 0) {
       RowConsts *rk = reinterpret_cast<RowConsts *>(top);
       k_at = (int)(top - el_sm);
       w_at = k_at + (int)sizeof(RowConsts) + (threadIdx.x >> 5) * en.row_bytes;
@@ -893,27 +885,23 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
         } else if constexpr (KIND == kRunChunks) {
           lean_chunks<double, FIXED>(sl, lp, c, ch, d.k, rank, n64);
         } else if constexpr (KIND == kRunMixed) {
-          lean_chunks_of_head<FIXED>(n, en.apu64, c, ch, d.k, rank, n64);
+          lean_chunks<float, FIXED>(sl, lp, c, ch, d.k, rank, n64);
         } else {
           const ElPlan pl{en.apu64, en.split64};
-          if (d.fp64) {
+          if (ROWS > 0 || !d.fp64) {
+            built64 = el_stage_of<double, float, kElFixed, false>(s64, c, g, pl, rank, n64, built64);
+          } else if constexpr (ROWS == 0) {
             if (c.cplx_h) built64 = el_stage_of<double, double, kElFixed, true>(s64, c, g, pl, rank, n64, built64);
             else built64 = el_stage_of<double, double, kElFixed, false>(s64, c, g, pl, rank, n64, built64);
-          } else {
-            built64 = el_stage_of<double, float, kElFixed, false>(s64, c, g, pl, rank, n64, built64);
           }
         }
       }
       if (do32) {
         const StageCommon &c = cs[1][q];
-        const int first = (threadIdx.x >> 5) * n32 + r32, stride = n32 * (kElThreads / 32);
-        if constexpr (KIND == kRunMixed) {
-          row_dispatch<1, kLeanMaxStates>(n, [&](auto N) { row_body<N.value>(k_at, w_at, c, (float)ch, first, stride); });
+        if constexpr (ROWS > 0) {
+          row_body<ROWS>(k_at, w_at, c, (float)ch, (threadIdx.x >> 5) * n32 + r32, n32 * (kElThreads / 32));
         } else if constexpr (KIND == kRunOther) {
-          if (rows)
-            row_dispatch<kLeanMaxStates + 1, kMaxStates>(n, [&](auto N) { row_body<N.value>(k_at, w_at, c, (float)ch, first, stride); });
-          else
-            built32 = el_stage_of<float, float, kElRowOrder, false>(s32, c, g, ElPlan{en.apu32, 1}, r32, n32, built32);
+          built32 = el_stage_of<float, float, kElRowOrder, false>(s32, c, g, ElPlan{en.apu32, 1}, r32, n32, built32);
         }
       }
       target += ncta;
