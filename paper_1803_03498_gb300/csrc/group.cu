@@ -123,22 +123,23 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   }
 
   int rc = HEOM_OK;
-  // small FP64 runs: whole steps in shared launches (resident.cuh), before the others' stages
-  std::vector<bool> done(n_runs, false);
+  // small FP64 runs: whole steps in shared launches (resident.cuh), before the others' stages; what a context too
+  // small for such a launch leaves of them is in `left` with the others' steps
+  std::vector<int64_t> left(n_steps, n_steps + n_runs);
   if (!capturing(gs)) {
     std::vector<heom_run *> small;
-    std::vector<int64_t> small_steps;
+    std::vector<int64_t> small_steps, before;
+    std::vector<int> who;
     for (int i = 0; i < n_runs; ++i) {
-      done[i] = !listed[i] && n_steps[i] > 0 && rv[i]->precision == HEOM_FP64 && el_small(rv[i]);
-      if (!done[i]) continue;
+      if (listed[i] || n_steps[i] == 0 || rv[i]->precision != HEOM_FP64 || !el_small(rv[i])) continue;
+      who.push_back(i);
       small.push_back(rv[i]);
       small_steps.push_back(n_steps[i]);
+      before.push_back(rv[i]->steps_done);
     }
     if (!small.empty()) rc = el_propagate(small.data(), (int)small.size(), h, small_steps.data(), obs_stride, gs);
-    if (rc == kElNoRoom) {
-      rc = HEOM_OK;
-      done.assign(n_runs, false);
-    }
+    if (rc == kElNoRoom) rc = HEOM_OK;
+    for (size_t k = 0; k < who.size(); ++k) left[who[k]] -= small[k]->steps_done - before[k];
   }
   // Each size class gets a stream of its own for the whole call (forked from and joined back into the
   // caller's stream): the classes' launch chains run side by side, while the stages of one class
@@ -149,7 +150,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   bool single = true;
   int n0 = -1;
   for (int i = 0; i < n_runs && single; ++i) {
-    if (n_steps[i] == 0 || done[i]) continue;
+    if (left[i] == 0) continue;
     if (n0 < 0) n0 = rv[i]->n;
     single = listed[i] && rv[i]->n == n0;
   }
@@ -188,11 +189,11 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   int64_t rebuilt_at = -1;
   for (int64_t s = 0; s < max_steps && rc == HEOM_OK; ++s) {
     bool change = rebuilt_at < 0;
-    for (int i = 0; i < n_runs && !change; ++i) change = listed[i] && n_steps[i] == s;
+    for (int i = 0; i < n_runs && !change; ++i) change = listed[i] && left[i] == s;
     if (change) {
       std::map<int, std::vector<int>> classes;  // n_states -> listed runs still stepping
       for (int i = 0; i < n_runs; ++i)
-        if (listed[i] && n_steps[i] > s) classes[rv[i]->n].push_back(i);
+        if (listed[i] && left[i] > s) classes[rv[i]->n].push_back(i);
       prep.clear();
       for (const auto &cl : classes) {
         cudaStream_t cs = gs;
@@ -263,7 +264,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       }
       // runs outside the work lists: their own launches, on the caller's stream
       for (int i = 0; i < n_runs && rc == HEOM_OK; ++i) {
-        if (listed[i] || done[i] || n_steps[i] <= s) continue;
+        if (listed[i] || left[i] <= s) continue;
         heom_run *r = rv[i];
         const HornerStage &hs = kHorner[st];
         cudaStream_t own = r->stream;
@@ -273,7 +274,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       }
     }
     for (int i = 0; i < n_runs && rc == HEOM_OK; ++i) {  // step counters and observable records
-      if (n_steps[i] <= s || done[i]) continue;
+      if (left[i] <= s) continue;
       heom_run *r = rv[i];
       ++r->steps_done;
       r->t_fs += h;

@@ -316,8 +316,8 @@ bool el_small(const heom_run *r) {
   return r->precision == HEOM_FP32_MIXED && !r->cplx_h && r->u_split > 0 && cost32(r) <= kElMaxCost32;
 }
 
-// A cooperative launch that this context cannot hold at once (fewer SMs than the device has): nothing was enqueued, and
-// the caller launches stage by stage.
+// A cooperative launch that this context cannot hold at once (fewer SMs than the device has): it was not enqueued, and the
+// caller takes the steps that the runs' counters still lack stage by stage.
 static bool no_room(cudaError_t e) {
   if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return false;
   cudaGetLastError();
@@ -446,7 +446,7 @@ static int propagate_form(int form, heom_run *const *runs, int n_runs, double h,
       void *args[] = {&L};
       cudaError_t ce = cudaLaunchCooperativeKernel(kernel, dim3(cta), dim3(threads), args, smem, s);
       if (ce == cudaSuccess) ce = cudaGetLastError();
-      if (no_room(ce) && at == 0 && b0 == 0) return kElNoRoom;
+      if (no_room(ce)) return kElNoRoom;
       if (ce != cudaSuccess) return cuda_fail("element run kernel launch", ce);
       for (size_t q = 0; q < in.size(); ++q) {
         heom_run *r = runs[in[q]];
@@ -462,7 +462,7 @@ static int propagate_form(int form, heom_run *const *runs, int n_runs, double h,
 }
 
 // Steps [done, done + steps[i]) of every run on stream s, as few launches as possible; the runs' counters
-// (steps_done, t_fs, records_host, launches) advance.
+// (steps_done, t_fs, records_host, launches) advance, also where it stops with kElNoRoom.
 int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
   std::vector<heom_run *> rs[kForms];
   std::vector<int64_t> st[kForms];
@@ -475,14 +475,10 @@ int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *ste
     rs[form].push_back(runs[i]);
     st[form].push_back(steps[i]);
   }
-  int n_done = 0;
   for (int form = 0; form < kForms; ++form) {
     if (rs[form].empty()) continue;
     const int rc = propagate_form(form, rs[form].data(), (int)rs[form].size(), h, st[form].data(), stride, s);
-    if (rc == kElNoRoom && n_done == 0) return rc;
-    if (rc == kElNoRoom) return cuda_fail("element run kernel launch", cudaErrorCooperativeLaunchTooLarge);
     if (rc != HEOM_OK) return rc;
-    ++n_done;
   }
   return HEOM_OK;
 }
@@ -547,7 +543,7 @@ int col_propagate(heom_run *r, double h, int64_t steps, int64_t stride, cudaStre
     void *args[] = {&a};
     cudaError_t e = cudaLaunchCooperativeKernel((const void *)col_run_kernel, dim3(a.hcta + c32), dim3(kColThreads), args, smem, s);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (no_room(e) && at == 0) return kElNoRoom;
+    if (no_room(e)) return kElNoRoom;
     if (e != cudaSuccess) return cuda_fail("column run kernel launch", e);
     if (stride > 0) r->records_host += (r->steps_done + a.steps) / stride - r->steps_done / stride;
     r->steps_done += a.steps;
