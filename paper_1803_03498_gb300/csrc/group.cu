@@ -123,58 +123,91 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   }
 
   int rc = HEOM_OK;
-  // small FP64 runs: whole steps in shared launches (resident.cuh), before the others' stages; what a context too
-  // small for such a launch leaves of them is in `left` with the others' steps
+  // small FP64 runs: whole steps in shared launches (resident.cuh)
   std::vector<int64_t> left(n_steps, n_steps + n_runs);
+  std::vector<ElShared> shared;
   if (!capturing(gs)) {
     std::vector<heom_run *> small;
-    std::vector<int64_t> small_steps, before;
-    std::vector<int> who;
+    std::vector<int64_t> small_steps;
+    bool others = false;
+    int sm_count = 1;
+    int64_t ctas = 0;
     for (int i = 0; i < n_runs; ++i) {
-      if (listed[i] || n_steps[i] == 0 || rv[i]->precision != HEOM_FP64 || !el_small(rv[i])) continue;
-      who.push_back(i);
+      if (n_steps[i] == 0) continue;
+      if (listed[i] || rv[i]->precision != HEOM_FP64 || !el_small(rv[i])) {
+        others = true;
+        continue;
+      }
+      ctas += el_ctas(rv[i]);
       small.push_back(rv[i]);
       small_steps.push_back(n_steps[i]);
-      before.push_back(rv[i]->steps_done);
+      left[i] = 0;
+      sm_count = rv[i]->sm_count;
     }
-    if (!small.empty()) rc = el_propagate(small.data(), (int)small.size(), h, small_steps.data(), obs_stride, gs);
-    if (rc == kElNoRoom) rc = HEOM_OK;
-    for (size_t k = 0; k < who.size(); ++k) left[who[k]] -= small[k]->steps_done - before[k];
+    // Beside other runs, small ones that are content with a CTA on every other SM stay there: on all slots they kept
+    // the others' stages waiting (680 ADOs of 7 states beside a mixed run of 11628: 7.1 ms for 60 steps, so 5.8,
+    // one after the other 7.1).  Larger ones take all slots: held to a quarter of them, 3060 ADOs beside four mixed runs
+    // took up to 14 ms against 11.
+    const int cap = others && ctas <= sm_count / 2 ? sm_count / 2 : 2 * sm_count;
+    if (!small.empty()) shared = el_split(small.data(), (int)small.size(), small_steps.data(), cap);
   }
-  // Each size class gets a stream of its own for the whole call (forked from and joined back into the
-  // caller's stream): the classes' launch chains run side by side, while the stages of one class
+  // Each size class and each kind of shared launches gets a stream of its own for the whole call (forked from and joined
+  // back into the caller's stream): their launch chains run side by side, while the stages of one class
   // follow each other.  A run keeps its class, so its launches stay in order.
-  std::vector<cudaStream_t> cls(kMaxStates + 1, nullptr);
+  std::vector<cudaStream_t> cls(kMaxStates + 1, nullptr), shs(shared.size(), nullptr);
   std::vector<cudaEvent_t> cls_ev;
-  // one size class and nothing else: its launches go straight to the caller's stream
-  bool single = true;
+  // one size class or kind and nothing else: its launches go straight to the caller's stream
+  bool any = false, single = shared.size() <= 1;
   int n0 = -1;
   for (int i = 0; i < n_runs && single; ++i) {
     if (left[i] == 0) continue;
+    any = true;
     if (n0 < 0) n0 = rv[i]->n;
     single = listed[i] && rv[i]->n == n0;
   }
-  // the stream of size class n in *out (the caller's stream, which may be the NULL stream, when the call
-  // has a single class)
-  auto class_stream = [&](int n, cudaStream_t *out) -> int {
+  if (any && !shared.empty()) single = false;
+  // a stream forked from the caller's in *out (the caller's, which may be the NULL stream, when the call
+  // needs only one)
+  auto fork_stream = [&](cudaStream_t *slot, cudaStream_t *out) -> int {
     *out = gs;
     if (single) return HEOM_OK;
-    if (!cls[n]) {
-      // the class streams take the caller's priority, so that a high-priority caller's ticks stay ahead
+    if (!*slot) {
+      // the forked streams take the caller's priority, so that a high-priority caller's ticks stay ahead
       // of other streams' launches when SM slots free up
       cudaEvent_t fe = nullptr;
       int prio = 0;
       cudaError_t ce = cudaStreamGetPriority(gs, &prio);
-      if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&cls[n], cudaStreamNonBlocking, prio);
+      if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(slot, cudaStreamNonBlocking, prio);
       if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&fe, cudaEventDisableTiming);
       if (ce == cudaSuccess) cls_ev.push_back(fe);
       if (ce == cudaSuccess) ce = cudaEventRecord(fe, gs);
-      if (ce == cudaSuccess) ce = cudaStreamWaitEvent(cls[n], fe, 0);
+      if (ce == cudaSuccess) ce = cudaStreamWaitEvent(*slot, fe, 0);
       if (ce != cudaSuccess) return cuda_fail("heom_group_propagate: class stream", ce);
     }
-    *out = cls[n];
+    *out = *slot;
     return HEOM_OK;
   };
+  // the caller's stream waits for what is on st so far
+  auto join_stream = [&](cudaStream_t st) -> int {
+    cudaEvent_t je = nullptr;
+    cudaError_t ce = cudaEventCreateWithFlags(&je, cudaEventDisableTiming);
+    if (ce == cudaSuccess) ce = cudaEventRecord(je, st);
+    if (ce == cudaSuccess) ce = cudaStreamWaitEvent(gs, je, 0);
+    if (je) cudaEventDestroy(je);
+    return ce == cudaSuccess ? HEOM_OK : cuda_fail("heom_group_propagate: class stream join", ce);
+  };
+  for (size_t k = 0; k < shared.size() && rc == HEOM_OK; ++k) {
+    ElShared &g = shared[k];
+    std::vector<int64_t> goal;
+    for (size_t q = 0; q < g.runs.size(); ++q) goal.push_back(g.runs[q]->steps_done + g.steps[q]);
+    cudaStream_t st = gs;
+    if ((rc = fork_stream(&shs[k], &st)) == HEOM_OK) rc = el_propagate(g, h, obs_stride, st);
+    if (rc != kElNoRoom) continue;
+    // a context too small for the launch: the steps that are left go with the others', after those enqueued
+    rc = st == gs ? HEOM_OK : join_stream(st);
+    for (size_t q = 0; q < g.runs.size(); ++q)
+      left[std::find(rv.begin(), rv.end(), g.runs[q]) - rv.begin()] = goal[q] - g.runs[q]->steps_done;
+  }
   // the work-list launches of one step, rebuilt only when a run's steps end: per class of equal
   // n_states and per batch of at most kListMaxRuns runs, the head and body launch of each stage
   struct Prepared {
@@ -187,6 +220,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
   };
   std::vector<Prepared> prep;
   int64_t rebuilt_at = -1;
+  max_steps = *std::max_element(left.begin(), left.end());
   for (int64_t s = 0; s < max_steps && rc == HEOM_OK; ++s) {
     bool change = rebuilt_at < 0;
     for (int i = 0; i < n_runs && !change; ++i) change = listed[i] && left[i] == s;
@@ -197,7 +231,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       prep.clear();
       for (const auto &cl : classes) {
         cudaStream_t cs = gs;
-        if ((rc = class_stream(cl.first, &cs)) != HEOM_OK) break;
+        if ((rc = fork_stream(&cls[cl.first], &cs)) != HEOM_OK) break;
         // FP64 heads: Hermitian runs and others take different kernels
         for (int herm = 0; herm < 2; ++herm) {
           std::vector<heom_run *> hr;
@@ -286,16 +320,13 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
       }
     }
   }
-  // join the class streams back into the caller's stream
-  for (int n = 0; n <= kMaxStates; ++n) {
-    if (!cls[n]) continue;
-    cudaEvent_t je = nullptr;
-    cudaError_t ce = cudaEventCreateWithFlags(&je, cudaEventDisableTiming);
-    if (ce == cudaSuccess) ce = cudaEventRecord(je, cls[n]);
-    if (ce == cudaSuccess) ce = cudaStreamWaitEvent(gs, je, 0);
-    if (je) cudaEventDestroy(je);
-    cudaStreamDestroy(cls[n]);  // released once its work is done
-    if (ce != cudaSuccess && rc == HEOM_OK) rc = cuda_fail("heom_group_propagate: class stream join", ce);
+  // join the forked streams back into the caller's stream
+  cls.insert(cls.end(), shs.begin(), shs.end());
+  for (cudaStream_t st : cls) {
+    if (!st) continue;
+    const int jr = join_stream(st);
+    if (rc == HEOM_OK) rc = jr;
+    cudaStreamDestroy(st);  // released once its work is done
   }
   for (cudaEvent_t fe : cls_ev) cudaEventDestroy(fe);
 

@@ -131,7 +131,14 @@ int col_propagate(heom_run *r, double h, int64_t steps, int64_t stride, cudaStre
 const GroupArgs *group_args_of(const heom_run *r);
 int el_group_args(heom_run *r, double h, cudaStream_t s);
 void head_plan(const heom_run *r, int *apu, int *splits, int *ctas);
-int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s);
+struct ElShared {  // runs that share launches of whole steps, and the CTAs of those
+  int form, cap;
+  std::vector<heom_run *> runs;
+  std::vector<int64_t> steps;
+};
+std::vector<ElShared> el_split(heom_run *const *runs, int n_runs, const int64_t *steps, int cap);
+int el_propagate(const ElShared &g, double h, int64_t stride, cudaStream_t s);
+int64_t el_ctas(const heom_run *r);  // CTAs that suit a small FP64 run
 
 // the launch-schedule autotuner (tuner.cu)
 extern std::atomic<int> g_autotune;  // timed launches per candidate at creation (0: off)

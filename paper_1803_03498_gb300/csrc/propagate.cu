@@ -276,7 +276,7 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
     // whole steps per launch; a captured or timed call, or a context too small for the launch, goes stage by stage
     const int64_t goal = r->steps_done + n_steps;
     const int rc = r->vec ? col_propagate(r, h, n_steps, obs_stride, r->stream)
-                          : el_propagate(&r, 1, h, &n_steps, obs_stride, r->stream);
+                          : el_propagate(el_split(&r, 1, &n_steps, 2 * r->sm_count)[0], h, obs_stride, r->stream);
     if (rc != kElNoRoom) return rc;
     n_steps = goal - r->steps_done;
   }

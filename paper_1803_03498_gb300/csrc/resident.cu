@@ -353,7 +353,12 @@ static const void *form_kernel(int form) {
   return k;
 }
 
-static int propagate_form(int form, heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
+// Every run of g by its number of steps on stream s, in as few launches as possible; the runs' counters
+// (steps_done, t_fs, records_host, launches) advance, also where it stops with kElNoRoom.
+int el_propagate(const ElShared &g, double h, int64_t stride, cudaStream_t s) {
+  const int form = g.form, n_runs = (int)g.runs.size(), cap = g.cap;
+  heom_run *const *runs = g.runs.data();
+  const int64_t *steps = g.steps.data();
   static std::atomic<bool> ready[kForms];
   const void *kernel = form_kernel(form);
   if (!kernel) {
@@ -367,7 +372,6 @@ static int propagate_form(int form, heom_run *const *runs, int n_runs, double h,
   }
   const bool kept_form = form < 2;
   const int threads = kept_form ? kLeanRunThreads : kElThreads;
-  const int sm_count = runs[0]->sm_count, cap = 2 * sm_count;  // 2 CTAs per SM (launch bounds; kElSmemMax)
   int64_t most = 0;
   for (int i = 0; i < n_runs; ++i) most = std::max(most, steps[i]);
   const int per_launch = std::min(kElMaxRuns, cap);  // a CTA for each run
@@ -461,26 +465,35 @@ static int propagate_form(int form, heom_run *const *runs, int n_runs, double h,
   return HEOM_OK;
 }
 
-// Steps [done, done + steps[i]) of every run on stream s, as few launches as possible; the runs' counters
-// (steps_done, t_fs, records_host, launches) advance, also where it stops with kElNoRoom.
-int el_propagate(heom_run *const *runs, int n_runs, double h, const int64_t *steps, int64_t stride, cudaStream_t s) {
-  std::vector<heom_run *> rs[kForms];
-  std::vector<int64_t> st[kForms];
-  int need[2] = {0, 0};  // CTAs that keep the runs without and with fixed point
-  for (int i = 0; i < n_runs; ++i)
-    if (run_lean(runs[i]) && runs[i]->precision == HEOM_FP64) need[form_of(runs[i], true)] += kept_ctas(runs[i]);
-  for (int i = 0; i < n_runs; ++i) {
-    int form = form_of(runs[i], true);
-    if (form < 2 && need[form] > 2 * runs[i]->sm_count) form = form_of(runs[i], false);
-    rs[form].push_back(runs[i]);
-    st[form].push_back(steps[i]);
+int64_t el_ctas(const heom_run *r) { return run_lean(r) ? kept_ctas(r) : 1 + (int64_t)(cost64(r) / (4 * kElGrain)); }
+
+// The runs by their form of launch, each with a share by cost of `cap` CTAs (at most 2 per SM: launch bounds and
+// kElSmemMax), so that launches on streams of their own fit the GPU beside each other.
+std::vector<ElShared> el_split(heom_run *const *runs, int n_runs, const int64_t *steps, int cap) {
+  std::vector<ElShared> out;
+  auto add = [&](int form, int i) {
+    for (ElShared &g : out)
+      if (g.form == form) {
+        g.runs.push_back(runs[i]);
+        g.steps.push_back(steps[i]);
+        return;
+      }
+    out.push_back(ElShared{form, 0, {runs[i]}, {steps[i]}});
+  };
+  for (int i = 0; i < n_runs; ++i) add(form_of(runs[i], true), i);
+  double total = 0;
+  for (int i = 0; i < n_runs; ++i) total += cost64(runs[i]) + cost32(runs[i]);
+  for (ElShared &g : out) {
+    double cost = 0;
+    int need = 0;  // CTAs that keep the runs
+    for (const heom_run *r : g.runs) {
+      cost += cost64(r) + cost32(r);
+      if (g.form < 2) need += kept_ctas(r);
+    }
+    g.cap = std::max(1, std::min(cap, (int)(cap * cost / total + 0.5)));
+    if (g.form < 2 && need > g.cap) g.form += 2;
   }
-  for (int form = 0; form < kForms; ++form) {
-    if (rs[form].empty()) continue;
-    const int rc = propagate_form(form, rs[form].data(), (int)rs[form].size(), h, st[form].data(), stride, s);
-    if (rc != HEOM_OK) return rc;
-  }
-  return HEOM_OK;
+  return out;
 }
 
 // ---- column-0 runs --------------------------------------------------------------------------------------
