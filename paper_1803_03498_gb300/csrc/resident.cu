@@ -330,6 +330,14 @@ static int kept_ctas(const heom_run *r) {
   return (int)((r->n_ado + a - 1) / a);
 }
 
+// ADOs per unit, at most `fit`, of a part of `ados` ADOs on `ctas` CTAs: every CTA gets the same number of units, none nearly
+// empty.  (Units as large as fit: 11628 non-Hermitian ADOs of 7 states were 364 units on 304 CTAs, two rounds for work of
+// little more than one; 467 us per step against 356 stage by stage before.)
+static int even_units(int64_t ados, int ctas, int fit) {
+  const int64_t per = (ados + ctas - 1) / ctas, rounds = (per + fit - 1) / fit;
+  return (int)((per + rounds - 1) / rounds);
+}
+
 // The forms of el_run_kernel (kind, fixed, states of the row form) and their kernels.
 constexpr int kFormOther = 4, kFormMixed = 8, kForms = kFormMixed + kMaxStates + 1;  // 0..3: kept, chunks; 8 + n: mixed
 static int form_of(const heom_run *r, bool kept) {
@@ -422,10 +430,9 @@ int el_propagate(const ElShared &g, double h, int64_t stride, cudaStream_t s) {
         e.cta0 = cta;
         e.hcta = h64;
         const size_t room = one && !fp64 ? kElSmemMax / 6 : kElSmemMax;
-        e.apu64 = (int)std::min<int64_t>((n64 + h64 - 1) / h64, fit_ados(r->n, pitch64, P, 8, true, room));
-        if (run_lean(r)) e.apu64 = (int)std::min<int64_t>((n64 + h64 - 1) / h64, lean_ados(r->n, threads));
+        e.apu64 = even_units(n64, h64, run_lean(r) ? lean_ados(r->n, threads) : fit_ados(r->n, pitch64, P, 8, true, room));
         e.split64 = n64 < h64 ? std::max(1, std::min(h64 / (int)n64, P / 64)) : 1;
-        e.apu32 = nb > 0 ? (int)std::min<int64_t>((nb + h32 - 1) / h32, fit_ados(r->n, r->Ep, P, 4, false, room)) : 1;
+        e.apu32 = nb > 0 ? even_units(nb, h32, fit_ados(r->n, r->Ep, P, 4, false, room)) : 1;
         longest = std::max(longest, one ? cost : std::max(cost64(r) / h64, cost32(r) / std::max(1, h32)));
         e.row_bytes = nb > 0 && r->herm ? row_bytes(r->n) : 0;
         const size_t m64 = run_lean(r) ? lean_smem_bytes(r->n, e.apu64, kept_form ? threads : 0)
