@@ -283,6 +283,14 @@ int row_bytes(int n) {
 // A CTA's share of one stage below which another CTA costs more (barrier, tile traffic) than it takes off.
 constexpr double kElGrain = 1500.0;
 
+// Whether one CTA takes a whole run: its barrier is then a __syncthreads.  The head and the body of a mixed run follow each
+// other there, so only the smallest stay in one (us per step in one CTA and in two: 2 states, 70 ADOs 31.7 and 25.5;
+// 3 states, 56 ADOs 26.2 and 21.7, from a coherence 48.2 and 39.5; 2 states, 6 ADOs 20.8 and 18.1).
+bool one_cta(const heom_run *r) {
+  const double cost = cost64(r) + cost32(r);
+  return cost <= (cost32(r) > 0 ? 0.3 : 2.0) * kElGrain;
+}
+
 struct ElShare {
   int n64, n32;  // CTAs of the FP64 part and of the body (1, 1: one CTA for both)
 };
@@ -292,7 +300,7 @@ ElShare share_of(const heom_run *r, int cap) {
   const double a = cost64(r), b = cost32(r);
   const int64_t n64 = r->precision == HEOM_FP64 ? r->n_ado : r->u_split, nb = r->n_ado - n64;
   const int P = el_pairs(r->n, r->herm);
-  if (cap <= 1 || a + b <= 2 * kElGrain) return ElShare{1, nb > 0 ? 1 : 0};
+  if (cap <= 1 || one_cta(r)) return ElShare{1, nb > 0 ? 1 : 0};
   // the most CTAs each part can use: an element kernel splits an FP64 ADO down to 64 pairs
   const double max64 = (double)n64 * (run_lean(r) ? 1 : std::max(1, P / 64)), max32 = (double)nb;
   double w64 = std::min(std::max(1.0, a / kElGrain), max64), w32 = nb > 0 ? std::min(std::max(1.0, b / kElGrain), max32) : 0.0;
@@ -399,7 +407,7 @@ int el_propagate(const ElShared &g, double h, int64_t stride, cudaStream_t s) {
           total += cost64(runs[i]) + cost32(runs[i]);
           if (kept_form) kept += kept_ctas(runs[i]);
           const ElShare w = share_of(runs[i], cap);
-          want += w.n64 == 1 && w.n32 <= 1 && cost64(runs[i]) + cost32(runs[i]) <= 2 * kElGrain ? 1 : w.n64 + w.n32;
+          want += one_cta(runs[i]) ? 1 : w.n64 + w.n32;
         }
       if (in.empty()) break;
       size_t smem = 0;
@@ -423,7 +431,7 @@ int el_propagate(const ElShared &g, double h, int64_t stride, cudaStream_t s) {
         // a kept run spreads until its CTAs have a warp for each partition of their SM (FP64 instructions of
         // one warp follow each other 64 clocks apart, whatever the other partitions do)
         const int64_t kept_h = std::min<int64_t>(r->n_ado, std::max<int64_t>(kept_ctas(r), std::min<int64_t>(mine, (r->n_ado * P + 127) / 128)));
-        const bool one = kept_form ? kept_h == 1 : mine <= 1 || cost <= 2 * kElGrain;
+        const bool one = kept_form ? kept_h == 1 : mine <= 1 || one_cta(r);
         const int h64 = kept_form ? (int)kept_h : one ? 1 : w.n64, h32 = one ? 1 : w.n32;
         ElEntry &e = L.e[L.nruns++];
         e.d = reinterpret_cast<const ElRunDesc *>(r->desc_dev);
