@@ -181,6 +181,9 @@ HEOM_DECLARE_LAUNCH(launch_stage_fp32_d)
 // Column-form FP64 stage kernel (stage_col.cuh) for Hermitian runs with a real H and 8 <= n <= 16:
 // every lane of a warp owns one column of one part of an ADO's result, so all 32 lanes do FP64 work.
 // Returns 1 when it does not cover n.
+constexpr bool col_covers(int n) { return n >= 8 && n <= 16; }
+constexpr int col_gcd(int a, int b) { return b == 0 ? a : col_gcd(b, a % b); }
+constexpr int col_passes(int n) { return 2 * n / col_gcd(2 * n, 32); }  // of 32 columns per warp chunk
 int launch_stage_col(const StageCommon &c, double ch, const double *term, const double *H, cudaStream_t st,
                      int sm_count);
 

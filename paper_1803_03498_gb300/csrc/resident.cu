@@ -318,9 +318,15 @@ ElShare share_of(const heom_run *r, int cap) {
 // Small hierarchies: their work of one stage, spread over the GPU, takes at most a few tens of microseconds.
 // FP64 runs of this size take the element kernels in every form of launch (the others the column kernel, where
 // it covers them); FP32 bodies get the same bits from the element and the row kernels.
+// Where the column kernel covers a run, it takes less per ADO but P passes for a warp's first chunk (P = 1 for 8 and 16 states,
+// 3 for 12, 7 for 14, 11 for 11), each about 1.1 us per state: the line is kElColPass P N.  Measured on both sides, us per step
+// whole / column: 8 states, 1287 ADOs 29 / 51, 12870 195 / 165; 10, 8008 192 / 264, 19448 436 / 345; 11, 12376 370 / 578, 31824
+// 1014 / 795; 12, 6188 201 / 216, 18564 614 / 487; 14, 11628 572 / 586, 38760 1955 / 1304; 16, 969 107 / 100, 4845 409 / 238.
+// Elsewhere stage launches of the same kernels come level at kElMaxCost64: 7 states, 19448 ADOs 218 / 228,
+// 31824 345 / 345; 18 states, 1330 ADOs 159 / 171, 7315 774 / 763.
 bool el_small(const heom_run *r) {
   if (r->vec || r->gen) return false;
-  if (r->precision == HEOM_FP64) return cost64(r) <= kElMaxCost64;
+  if (r->precision == HEOM_FP64) return cost64(r) <= (r->herm && !r->cplx_h && col_covers(r->n) ? kElColPass * col_passes(r->n) * r->n : kElMaxCost64);
   return r->precision == HEOM_FP32_MIXED && !r->cplx_h && r->u_split > 0 && cost32(r) <= kElMaxCost32;
 }
 

@@ -46,8 +46,6 @@
 
 namespace heom {
 
-__host__ __device__ constexpr int col_gcd(int a, int b) { return b == 0 ? a : col_gcd(b, a % b); }
-
 // Most ADOs of C columns that one pass of 32 consecutive columns touches, over the P passes of a chunk.
 __host__ __device__ constexpr int col_ring(int C, int P) {
   int m = 1;
@@ -62,7 +60,8 @@ template <int N>
 struct ColShape {
   static constexpr int C = 2 * N;                  // columns per ADO (both parts)
   static constexpr int G = 32 / col_gcd(C, 32);    // ADOs per warp chunk
-  static constexpr int P = C * G / 32;             // passes of 32 columns per chunk
+  static constexpr int P = col_passes(N);          // passes of 32 columns per chunk
+  static_assert(P * 32 == C * G, "whole passes");
   static constexpr int E = N * N;
   static constexpr int RING = col_ring(C, P);      // Q slots: the ADOs one pass touches (N = 14: 2)
   static constexpr int RB = 12;                    // link records per batch and finalising ADO
