@@ -25,7 +25,7 @@ SOURCES = (["hierarchy.cpp", "heom_abi.cu", "propagate.cu", "tuner.cu", "batch.c
            + ["stage_tc_a.cu", "stage_tc_b.cu", "vec_stage_g1.cu", "vec_stage_g2.cu", "vec_stage_g4.cu",
               "stage_col.cu",
               "stage_list_a.cu", "stage_list_b.cu", "stage_list_c.cu", "group.cu"]
-           + [f"run_mixed_{g}.cu" for g in "abcd"])
+           + [f"run_mixed_{g}.cu" for g in "abc"])
 HEADERS = ["hierarchy.h", "heom_internal.h", "heom_run.h", "stage_kernel.cuh", "stage_tc.cuh", "vec_kernel.cuh", "resident.cuh", "column_run.cuh", "lean.cuh", "fixed_point.cuh", "record.cuh",
            "stage_col.cuh", "stage_list.cuh"]
 

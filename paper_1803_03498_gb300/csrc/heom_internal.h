@@ -238,7 +238,6 @@ struct ElEntry {
 const void *mixed_run_kernel_a(int n);
 const void *mixed_run_kernel_b(int n);
 const void *mixed_run_kernel_c(int n);
-const void *mixed_run_kernel_d(int n);
 constexpr int kElMaxRuns = 256;  // runs per launch (kernel parameters: about 10 KB)
 struct ElList {
   ElEntry e[kElMaxRuns];

@@ -123,6 +123,7 @@ inline double horner_c(int q, double h) { return q == 0 ? h / 4 : q == 1 ? h / 3
 constexpr double kElMaxCost64 = 1.6e7;  // cycles of one stage on one SM (see el_small)
 constexpr double kElColPass = 2.2e5;    // the same per state and pass of the column kernel
 constexpr double kElMaxCost32 = 1.5e6;
+constexpr int kElMaxRows = 18;          // states of a Hermitian FP32 body in a launch of whole steps
 constexpr int kElNoRoom = 1;  // el_propagate, col_propagate: the context cannot hold a launch (steps_done: how far each run is)
 ElConsts el_consts_of(const heom_run *r);
 int el_upload(heom_run *r);

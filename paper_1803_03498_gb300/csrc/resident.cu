@@ -305,8 +305,10 @@ ElShare share_of(const heom_run *r, int cap) {
   const double max64 = (double)n64 * (run_lean(r) ? 1 : std::max(1, P / 64)), max32 = (double)nb;
   double w64 = std::min(std::max(1.0, a / kElGrain), max64), w32 = nb > 0 ? std::min(std::max(1.0, b / kElGrain), max32) : 0.0;
   if (w64 + w32 > cap) {
+    // a head keeps the CTAs that it can use, up to a quarter: an ADO of 17 to 22 states takes one about 10 us, so
+    // two after each other in a CTA hold the body's CTAs at the barrier
     const double f = cap / (a + b);
-    w64 = std::max(1.0, std::min(max64, a * f));
+    w64 = std::max(1.0, nb > 0 ? std::min(w64, std::max(a * f, 0.25 * cap)) : std::min(max64, a * f));
     if (nb > 0) w32 = std::max(1.0, std::min(max32, cap - std::floor(w64)));
     w64 = std::min(max64, cap - std::floor(w32));
   }
@@ -324,10 +326,16 @@ ElShare share_of(const heom_run *r, int cap) {
 // 1014 / 795; 12, 6188 201 / 216, 18564 614 / 487; 14, 11628 572 / 586, 38760 1955 / 1304; 16, 969 107 / 100, 4845 409 / 238.
 // Elsewhere stage launches of the same kernels come level at kElMaxCost64: 7 states, 19448 ADOs 218 / 228,
 // 31824 345 / 345; 18 states, 1330 ADOs 159 / 171, 7315 774 / 763.
+// Mixed runs, whole steps / stage launches: up to kElMaxCost32 (about 6400 ADOs of 7 or 8 states, 3600 of 12) 7 states, 6435 ADOs
+// 33 / 42; 8, 6435 34 / 37; 10, 3003 32 / 42; 13, 2380 36 / 50; from a coherence 7, 3432 57 / 66, 6435 87 / 66.  From 16 states on the row
+// form spills at this kernel's 128 registers, and the lines lie lower: 16 states, 153 ADOs 35 / 42, 969 52 / 46; 17, 171 37 / 45,
+// 630 52 / 51 (a third of the limit); 19, 210 50 / 49; 22, 276 62 / 50 (from 19 on only heads without a body).
 bool el_small(const heom_run *r) {
   if (r->vec || r->gen) return false;
   if (r->precision == HEOM_FP64) return cost64(r) <= (r->herm && !r->cplx_h && col_covers(r->n) ? kElColPass * col_passes(r->n) * r->n : kElMaxCost64);
-  return r->precision == HEOM_FP32_MIXED && !r->cplx_h && r->u_split > 0 && cost32(r) <= kElMaxCost32;
+  if (r->precision != HEOM_FP32_MIXED || r->cplx_h || r->u_split <= 0) return false;
+  if (r->n_ado == r->u_split || !r->herm) return cost32(r) <= kElMaxCost32;
+  return r->n <= kElMaxRows && cost32(r) <= (r->n >= 16 ? kElMaxCost32 / 3 : kElMaxCost32);
 }
 
 // A cooperative launch that this context cannot hold at once (fewer SMs than the device has): it was not enqueued, and the
@@ -353,10 +361,11 @@ static int even_units(int64_t ados, int ctas, int fit) {
 }
 
 // The forms of el_run_kernel (kind, fixed, states of the row form) and their kernels.
-constexpr int kFormOther = 4, kFormMixed = 8, kForms = kFormMixed + kMaxStates + 1;  // 0..3: kept, chunks; 8 + n: mixed
+// 0..3: kept, chunks; 5: mixed without a body; 8 + n: mixed of n states
+constexpr int kFormOther = 4, kFormHead = 5, kFormMixed = 8, kForms = kFormMixed + kElMaxRows + 1;
 static int form_of(const heom_run *r, bool kept) {
-  if (r->precision != HEOM_FP64) return r->herm ? kFormMixed + r->n : kFormOther;
   if (!run_lean(r)) return kFormOther;
+  if (r->precision != HEOM_FP64) return r->n <= kElMaxRows ? kFormMixed + r->n : kFormHead;
   return (kept ? 0 : 2) + (lean_fixed(r->n, r->n_ado) ? 1 : 0);
 }
 static const void *form_kernel(int form) {
@@ -366,12 +375,12 @@ static const void *form_kernel(int form) {
     case 2: return (const void *)el_run_kernel<kRunChunks, false, 0>;
     case 3: return (const void *)el_run_kernel<kRunChunks, true, 0>;
     case kFormOther: return (const void *)el_run_kernel<kRunOther, true, 0>;
+    case kFormHead: return (const void *)el_run_kernel<kRunMixed, true, 0>;
   }
   const int n = form - kFormMixed;
   const void *k = mixed_run_kernel_a(n);
   if (!k) k = mixed_run_kernel_b(n);
   if (!k) k = mixed_run_kernel_c(n);
-  if (!k) k = mixed_run_kernel_d(n);
   return k;
 }
 

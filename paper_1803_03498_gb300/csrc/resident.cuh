@@ -842,7 +842,7 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
       top = s64.end;
       el_consts<double>(s64, d.k, n, d.c.herm, true, 0.0, 0.0);
       __syncthreads();
-      if (ROWS == 0 && d.c.cplx_h) el_fix_consts<true>(s64, n);
+      if (d.c.cplx_h) el_fix_consts<true>(s64, n);
       else el_fix_consts<false>(s64, n);
     }
   }
@@ -888,11 +888,11 @@ __global__ void __launch_bounds__(KIND == kRunKept ? kLeanRunThreads : kElThread
           lean_chunks<float, FIXED>(sl, lp, c, ch, d.k, rank, n64);
         } else {
           const ElPlan pl{en.apu64, en.split64};
-          if (ROWS > 0 || !d.fp64) {
-            built64 = el_stage_of<double, float, kElFixed, false>(s64, c, g, pl, rank, n64, built64);
-          } else if constexpr (ROWS == 0) {
+          if (d.fp64) {
             if (c.cplx_h) built64 = el_stage_of<double, double, kElFixed, true>(s64, c, g, pl, rank, n64, built64);
             else built64 = el_stage_of<double, double, kElFixed, false>(s64, c, g, pl, rank, n64, built64);
+          } else {
+            built64 = el_stage_of<double, float, kElFixed, false>(s64, c, g, pl, rank, n64, built64);
           }
         }
       }

@@ -1,4 +1,4 @@
-// Launches of whole steps of mixed runs, n_states 15..19.
+// Launches of whole steps of mixed runs, n_states 15..18.
 #include "resident.cuh"
 
 namespace heom {
@@ -9,7 +9,6 @@ const void *mixed_run_kernel_c(int n) {
     case 16: return (const void *)el_run_kernel<kRunMixed, true, 16>;
     case 17: return (const void *)el_run_kernel<kRunMixed, true, 17>;
     case 18: return (const void *)el_run_kernel<kRunMixed, true, 18>;
-    case 19: return (const void *)el_run_kernel<kRunMixed, true, 19>;
     default: return nullptr;
   }
 }
