@@ -290,7 +290,7 @@ extern "C" int heom_group_propagate(heom_run *const *runs, int n_runs, double dt
           p.H.stage = st;
           p.H.ch = horner_c(st, h);
         }
-        if (p.head ? launch_head_list(p.H, p.stream, p.sm_count) : launch_stage_list(p.n, p.L[st], p.stream, p.sm_count)) {
+        if (p.head ? launch_head_list(p.H, p.stream) : launch_stage_list(p.n, p.L[st], p.stream, p.sm_count)) {
           rc = HEOM_E_CUDA;
           break;
         }

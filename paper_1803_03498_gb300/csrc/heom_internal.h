@@ -275,7 +275,7 @@ struct HeadList {
   int stage;   // 0..3
   double ch;
 };
-int launch_head_list(const HeadList &L, cudaStream_t st, int sm_count);
+int launch_head_list(const HeadList &L, cudaStream_t st);
 
 // The FP32 body of a mixed run on the row kernels (stage_kernel.cuh).
 int launch_stage(const StageCommon &c, double ch, const double *term, const double *H,

@@ -50,8 +50,8 @@ struct heom_run {
   bool cplx_h = false;
   bool herm = false;                 // every ADO Hermitian (Hermitian H and data; paper gauge)
   bool vec = false;                  // every ADO in the coherence block |a><0|: stored as its column 0
-  bool gen = false;                  // general stage kernel (bath masks, laser field, > 24 states)
-  std::vector<double> T;             // [n][n] terminator rate of each element (general kernel)
+  bool gen = false;                  // general run: element kernels (bath masks, laser field, > 24 states)
+  std::vector<double> T;             // [n][n] terminator rate of each element (general runs)
   bool has_field = false;            // laser field set (heom_run_set_field): classic four-copy RK4
   std::vector<double> mup;           // [n][n] M+
   double famp = 0, ftc = 0, fsig = 1, fphase = 0, fdet = 0;  // rad/fs, fs, fs, rad, rad/fs

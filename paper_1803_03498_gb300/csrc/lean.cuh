@@ -8,15 +8,17 @@
 // tiles' scales, every thread writes its element and its mirror as limbs to shared memory, and while
 // the neighbour elements of up to four links are on their way it forms the commutator there.  FP64 instructions
 // (18.7 clocks per warp and SM) remain for decay, links and the RK4 combination: about 4 + 4 per link slot.
-// Measured, FP64 runs of 100 steps, us per step (row kernels before): 3060 ADOs of 7 x 7 99.8 -> 35.1, 680 of them 82.5 ->
-// 23.8, 435 of 14 x 14 464 -> 30.9, 1771 of 10 x 10 266 -> 66.
+// Measured, FP64 runs, us per step (row kernels before): 1716 ADOs of 7 x 7 69.5 -> 27.0, 330 of them 65.8 -> 19.1, 680 of
+// 14 x 14 393 -> 38.9, 3003 of 10 x 10 230 -> 84.
 #pragma once
 
 namespace heom {
 
 constexpr int kLeanMaxStates = 22;  // 253 pairs: one ADO fits a CTA of 256 threads
 constexpr int kLeanThreads = 256;   // stage kernel, and CTAs of mixed runs
-constexpr int kLeanRunThreads = 320;  // CTAs that keep FP64 runs: 2 per SM hold the 3060 ADOs of 7 states
+// CTAs that keep FP64 runs: more ADOs in each than with 256 threads, so that larger runs still fit (680 ADOs of 14 states
+// 38.9 us per step against 65.9, 2002 of 9 37 against 59), and more warps for the smallest (120 of 3 states 14.5 / 17.7)
+constexpr int kLeanRunThreads = 320;
 constexpr int kLeanSlots = 4;       // link slots in registers (stages); more are read in a loop
 constexpr int kLeanKept = 6;        // the same of CTAs that keep their ADOs
 
@@ -27,13 +29,16 @@ __host__ __device__ inline int lean_ados(int n, int threads) {
 }
 
 // Whether the commutator of a part of `ados` ADOs runs in fixed point.  An FP64 FMA holds its SM partition for 64
-// clocks whether one warp or many wait, so with few warps per SM 4 n of them per pair are as fast as the integer path
-// (7 states, 680 ADOs: 1800 clocks against 3800), and only the pipe's throughput counts from about 200 pairs per
-// SM on or where one ADO fills it.  A property of the run: every form of launch decides alike.
+// clocks whether one warp or many wait, so with few warps per SM 4 n of them per pair are as fast as the integer path,
+// and only the pipe's throughput counts from about 200 pairs per SM on or where one ADO fills it.  Measured, us per
+// step, FMAs / fixed point: 6 states, 19404 pairs 18.3 / 19.2, 36036 27.7 / 24.1; 7, 9240 19.0 / 19.8, 48048 33.4 / 27.0; 8, 17820
+// 19.6 / 21.0, 46332 33.2 / 27.1; 9, 2475 20.1 / 21.0, 32175 30.9 / 25.5; 12, 7098 21.7 / 23.4, 35490 34.4 / 28.2; 14, 1575
+// 25.7 / 23.6; 4 states, 12870 21.4 / 23.2.  A property of the run: every form of launch decides alike.
 __host__ __device__ inline bool lean_fixed(int n, int64_t ados) {
   return n >= 9 || (n >= 5 && ados * (n * (n + 1) / 2) >= 32768);
 }
-// The same for the head of a mixed run: its 1 + n_modes ADOs (at most 256) never reach the second line.
+// The same for the head of a mixed run: its 1 + n_modes ADOs (at most 256) never reach the second line.  Of one step, 8 states, 165
+// ADOs 27.7 / 28.0; 9, 715 32.6 / 32.3; 10, 1001 33.8 / 31.6; 12, 455 31.0 / 32.5, 1820 41.7 / 37.2.
 __host__ __device__ constexpr bool lean_head_fixed(int n) { return n >= 9; }
 
 // Shared memory: limbs of H and of the tiles, T, scale keys (two sets), link ranges; and for resident CTAs the

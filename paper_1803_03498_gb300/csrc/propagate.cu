@@ -1,4 +1,4 @@
-// C ABI of libheom, part 2: the RK4 driver.  Stage launches (head, body, general kernel), the laser
+// C ABI of libheom, part 2: the RK4 driver.  Stage launches (head, body, general runs), the laser
 // field's H(t), Horner and classic RK4 steps, kernel timing, observables and one RHS evaluation.
 #include <cuda_runtime.h>
 

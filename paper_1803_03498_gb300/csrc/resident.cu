@@ -138,9 +138,7 @@ int launch_el_stage(int kind, const ElStageArgs &in, const double *mup, cudaStre
   }
 }
 
-int launch_head_list(const HeadList &in, cudaStream_t st, int sm_count) {
-  (void)sm_count;
-  HeadList L = in;
+int launch_head_list(const HeadList &L, cudaStream_t st) {
   const bool lean = lean_covers(L.n, L.herm, 0, false);
   const int ctas = L.cta0[L.nruns];
   if (ctas <= 0) return 0;

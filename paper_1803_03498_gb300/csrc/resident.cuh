@@ -8,10 +8,10 @@
 // (both: 2 Re R; see LinkRec).  So a thread computes one element -- for a Hermitian run one pair
 // (i <= j), whose mirror element it also writes, half the work and exactly Hermitian results -- with
 // its neighbour loads independent of each other: no chain from link to link, which is what bound the
-// row kernel at these sizes (one warp-synchronised step per link; 24 us per launch for 3060 FP64 ADOs
+// FP64 row kernels once used at these sizes (one warp-synchronised step per link; 24 us per launch for 3060 ADOs
 // of 7 x 7, 18.7 us for 680, 58 us for the 20 FP64 head ADOs of a 19-state run).  Pairs of consecutive
 // ADOs are numbered through, so every lane has work for every n_states, and the pairs of one ADO can be
-// split over CTAs on different SMs: GB300's FP64 pipe (2 FMAs per clock per SM) bounds these kernels, and
+// split over CTAs on different SMs: GB300's FP64 pipe (18.7 clocks per warp FMA and SM) bounds these kernels, and
 // the few FP64 head ADOs of a mixed run (1 + M of them) then use the pipes of all SMs.
 //
 // Two forms of launch run the same code, so results do not depend on the form:
@@ -559,9 +559,9 @@ static_assert(kElThreads == kLeanThreads, "el_run_kernel runs both");
 // el_run_kernel has few chunks per stage, and the other warps of the SM cover its loads.
 template <int N>
 struct RowSmem {
-  using S = StageShape<N, float, float>;
+  using S = StageShape<N>;
   static constexpr int tile = 0;
-  static constexpr int rec = (S::A * S::EpBody * 8 + 15) & ~15;
+  static constexpr int rec = (S::A * S::Ep * 8 + 15) & ~15;
   static constexpr int gbuf = rec + 2 * S::RC * 16;
   static constexpr int tb = gbuf + ((S::RC * 2 * N * 8 + 15) & ~15);
   static constexpr int total = tb + 64;
@@ -575,9 +575,9 @@ struct RowConsts {
 // compiler can see to be shared: through generic pointers the same code ran 3.5 times slower).
 template <int N>
 __device__ __forceinline__ void row_body(int k_at, int w_at, const StageCommon &cr, float ch, int first, int nwarps) {
-  using S = StageShape<N, float, float>;
+  using S = StageShape<N>;
   using W = RowSmem<N>;
-  constexpr int A = S::A, EPO = S::EpBody;
+  constexpr int A = S::A, EPO = S::Ep;
   extern __shared__ __align__(16) unsigned char el_sm[];
   const RowConsts &k = *reinterpret_cast<const RowConsts *>(el_sm + k_at);
   unsigned char *wb = el_sm + w_at;
@@ -603,7 +603,7 @@ __device__ __forceinline__ void row_body(int k_at, int w_at, const StageCommon &
     cp_async_commit();
     cp_async_wait<0>();
     __syncwarp();
-    issue_gathers<N, float, float>(c, rec, nrec, gbuf, lane);
+    issue_gathers<N>(c, rec, nrec, gbuf, lane);
     const bool active = lane_ok && la < cnt;
     float rr[N], ri[N];
     if (active) {
@@ -653,8 +653,8 @@ __device__ __forceinline__ void row_body(int k_at, int w_at, const StageCommon &
     }
     cp_async_wait<0>();
     __syncwarp();
-    owner_apply<N, float, float>(c, recs, c.rec_split, rec, gbuf, wb + W::tb, lo, hi, nrec, cap, u0, lane, rr, ri);
-    owner_combine<N, float, float>(active, la, li, zt_all, rr, ri);
+    owner_apply<N>(c, recs, c.rec_split, rec, gbuf, wb + W::tb, lo, hi, nrec, cap, u0, lane, rr, ri);
+    owner_combine<N>(active, la, li, zt_all, rr, ri);
     __syncwarp();
     // out = y + ch R, 16 bytes per access
     const int64_t at = (int64_t)(u0 - c.u_split) * EPO;
@@ -687,11 +687,10 @@ __global__ void __launch_bounds__(kElThreads, 2) el_stage_kernel(const __grid_co
   extern __shared__ __align__(16) unsigned char el_sm[];
   constexpr bool OWN_HEAD = sizeof(CT) == 8 && sizeof(BT) == 4;
   const StageCommon &c = a.c;
-  constexpr bool general = FORM != kElRowOrder;
-  const ElSmem<CT> s = el_carve<CT>(el_sm, c.n, a.apu, OWN_HEAD ? c.E : c.Ep, el_pairs(c.n, c.herm), general);
+  const ElSmem<CT> s = el_carve<CT>(el_sm, c.n, a.apu, OWN_HEAD ? c.E : c.Ep, el_pairs(c.n, c.herm), true);
   ElConsts k = a.k;
   if constexpr (CPLX) k.mup = field ? m.v : nullptr;
-  el_consts<CT>(s, k, c.n, c.herm, general, a.gr, a.gi);
+  el_consts<CT>(s, k, c.n, c.herm, true, a.gr, a.gi);
   __syncthreads();
   if constexpr (FORM == kElFixed) {
     el_fix_consts<CPLX>(s, c.n);

@@ -16,7 +16,7 @@ int launch_stage_col(const StageCommon &c, double ch, const double *term, const 
     case 15: return launch_col<15>(c, ch, term, H, st, sm_count);
     case 16: return launch_col<16>(c, ch, term, H, st, sm_count);
     default:
-      return 1;  // not covered: the row-form stage kernel runs
+      return 1;  // not covered: the element kernels run
   }
 }
 

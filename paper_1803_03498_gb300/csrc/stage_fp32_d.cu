@@ -6,12 +6,12 @@ namespace heom {
 int launch_stage_fp32_d(const StageCommon &c, double ch, const double *term, const double *H, const double *Hi,
                        cudaStream_t st, int sm_count) {
   switch (c.n) {
-    case 19: return launch_n<19, float, float>(c, ch, term, H, Hi, st, sm_count);
-    case 20: return launch_n<20, float, float>(c, ch, term, H, Hi, st, sm_count);
-    case 21: return launch_n<21, float, float>(c, ch, term, H, Hi, st, sm_count);
-    case 22: return launch_n<22, float, float>(c, ch, term, H, Hi, st, sm_count);
-    case 23: return launch_n<23, float, float>(c, ch, term, H, Hi, st, sm_count);
-    case 24: return launch_n<24, float, float>(c, ch, term, H, Hi, st, sm_count);
+    case 19: return launch_n<19>(c, ch, term, H, Hi, st, sm_count);
+    case 20: return launch_n<20>(c, ch, term, H, Hi, st, sm_count);
+    case 21: return launch_n<21>(c, ch, term, H, Hi, st, sm_count);
+    case 22: return launch_n<22>(c, ch, term, H, Hi, st, sm_count);
+    case 23: return launch_n<23>(c, ch, term, H, Hi, st, sm_count);
+    case 24: return launch_n<24>(c, ch, term, H, Hi, st, sm_count);
     default:
       return 1;  // not in this translation unit
   }

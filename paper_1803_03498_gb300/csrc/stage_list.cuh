@@ -13,8 +13,8 @@
 namespace heom {
 
 template <int N>
-__global__ void __launch_bounds__(StageShape<N, float, float>::WARPS * 32) stage_list_kernel(const __grid_constant__ ListLaunch L) {
-  using S = StageShape<N, float, float>;
+__global__ void __launch_bounds__(StageShape<N>::WARPS * 32) stage_list_kernel(const __grid_constant__ ListLaunch L) {
+  using S = StageShape<N>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ GroupArgs ga;
   static_assert(sizeof(GroupArgs) % 16 == 0, "16-byte copies");
@@ -35,14 +35,14 @@ __global__ void __launch_bounds__(StageShape<N, float, float>::WARPS * 32) stage
     __syncthreads();
     const int n_chunks = (ga.c.u_end - ga.c.u_begin + S::A - 1) / S::A;
     const int c0 = (it - L.item0[lo]) * L.cpi;
-    stage_chunks<N, float, float, false>(ga, smem_raw, c0 + (int)(threadIdx.x >> 5), S::WARPS, min(n_chunks, c0 + L.cpi));
+    stage_chunks<N, false>(ga, smem_raw, c0 + (int)(threadIdx.x >> 5), S::WARPS, min(n_chunks, c0 + L.cpi));
   }
 }
 
 template <int N>
 int launch_list_n(const ListLaunch &L, cudaStream_t st, int sm_count) {
-  constexpr int WARPS = StageShape<N, float, float>::WARPS;
-  const size_t smem = (size_t)WARPS * WarpSmem<N, float, float>::total;
+  constexpr int WARPS = StageShape<N>::WARPS;
+  const size_t smem = (size_t)WARPS * WarpSmem<N>::total;
   static int per_sm = 0;
   if (per_sm == 0) {
     cudaError_t e = cudaFuncSetAttribute(stage_list_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -167,11 +167,11 @@ struct TcSmem {
 template <int N>
 __global__ void __launch_bounds__(kTcWarps * 32, HEOM_TC_MIN_BLOCKS) stage_tc_kernel(const __grid_constant__ StageArgs<float> a) {
   static_assert(N >= 1 && N <= kTcK, "the tensor-core form covers n_states <= 16");
-  using S = StageShape<N, float, float, kTcRC>;
-  using W = WarpSmem<N, float, float, kTcRC>;
+  using S = StageShape<N, kTcRC>;
+  using W = WarpSmem<N, kTcRC>;
   using C2 = float2;
   using R = LinkRec<float>;
-  constexpr int A = S::A, EPO = S::EpOwn;
+  constexpr int A = S::A, EPO = S::Ep;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StageCommon &c = a.c;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, HEOM_TC_MIN_BLOCKS) stage_tc_ke
   if (first < n_chunks) {
     const int u0 = c.u_begin + first * A;
     const int cnt = min(A, c.u_end - u0);
-    issue_tiles<N, float, float>(zin_own, own0, u0, cnt, wb + W::tile0, lane, same_y);
+    issue_tiles<N>(zin_own, own0, u0, cnt, wb + W::tile0, lane, same_y);
     const int64_t lo = __shfl_sync(0xffffffffu, off_cur, 0), hi = __shfl_sync(0xffffffffu, off_cur, cnt);
     const int nr = heom_rec_batch(c.err, lo, (int)min(hi - lo, (int64_t)cap), rbase, c.n_recs);
     warp_copy16(wb + W::rec0, recs + (lo - rbase), nr * (int)sizeof(R), lane);
@@ -258,13 +258,13 @@ __global__ void __launch_bounds__(kTcWarps * 32, HEOM_TC_MIN_BLOCKS) stage_tc_ke
     if (nx < n_chunks) {
       const int v0 = c.u_begin + nx * A;
       const int vcnt = min(A, c.u_end - v0);
-      issue_tiles<N, float, float>(zin_own, own0, v0, vcnt, wb + (b ? W::tile0 : W::tile1), lane, same_y);
+      issue_tiles<N>(zin_own, own0, v0, vcnt, wb + (b ? W::tile0 : W::tile1), lane, same_y);
       const int64_t lo = __shfl_sync(0xffffffffu, off_nxt, 0), hi = __shfl_sync(0xffffffffu, off_nxt, vcnt);
       const int nr = heom_rec_batch(c.err, lo, (int)min(hi - lo, (int64_t)cap), rbase, c.n_recs);
       warp_copy16(wb + (b ? W::rec0 : W::rec1), recs + (lo - rbase), nr * (int)sizeof(R), lane);
     }
     cp_async_commit();
-    if (valid && kYSmem && has_y) issue_tiles<N, float, float>(y_own, own0, u0, cnt, ybuf, lane);
+    if (valid && kYSmem && has_y) issue_tiles<N>(y_own, own0, u0, cnt, ybuf, lane);
     cp_async_commit();
     cp_async_wait<2>();  // this chunk's tiles and first records have landed
     __syncwarp();
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, HEOM_TC_MIN_BLOCKS) stage_tc_ke
 
     // while the tensor cores run: neighbour gathers, half the decay and terminator (Q + Q^dagger
     // restores the rest), the links
-    if (valid) issue_gathers<N, float, float>(c, rec, nrec, gbuf, lane);
+    if (valid) issue_gathers<N>(c, rec, nrec, gbuf, lane);
     float rr[N], ri[N];
     if (active) {
       const float gsv = (float)c.gsum[u0 + la];
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, HEOM_TC_MIN_BLOCKS) stage_tc_ke
     cp_async_wait<0>();  // gathers, y and the next chunk's copies have landed
     __syncwarp();
     if (valid)
-      owner_apply<N, float, float>(c, recs, rbase, rec, gbuf, wb + W::tb, lo, hi, nrec, cap, u0, lane, rr, ri);
+      owner_apply<N>(c, recs, rbase, rec, gbuf, wb + W::tb, lo, hi, nrec, cap, u0, lane, rr, ri);
 
     {  // bounded wait for this round's MMAs
       const long long t0 = clock64();
@@ -371,9 +371,9 @@ __global__ void __launch_bounds__(kTcWarps * 32, HEOM_TC_MIN_BLOCKS) stage_tc_ke
       }
     }
     if (valid) {
-      owner_combine<N, float, float>(active, la, li, zt_all, rr, ri);
+      owner_combine<N>(active, la, li, zt_all, rr, ri);
       __syncwarp();
-      store_chunk<N, float, float>(out_own, y_own, own0, u0, cnt, has_y, a.ch, zt_all, ybuf, lane);
+      store_chunk<N>(out_own, y_own, own0, u0, cnt, has_y, a.ch, zt_all, ybuf, lane);
     }
     __syncwarp();  // this tile buffer, record buffer and ybuf are reused by later chunks
     off_cur = off_nxt;
@@ -410,7 +410,7 @@ int launch_tc(const StageCommon &c, double ch, const double *term, const double 
   }
   for (int i = 0; i < c.n; ++i)
     for (int j = 0; j < c.n; ++j) a.H[i * kMaxStates + j] = (float)H[i * c.n + j];
-  const size_t smem = (size_t)TcSmem::total + (size_t)kTcWarps * WarpSmem<N, float, float, kTcRC>::total;
+  const size_t smem = (size_t)TcSmem::total + (size_t)kTcWarps * WarpSmem<N, kTcRC>::total;
   // CTAs per SM from the kernel's registers, shared memory and tensor memory (the occupancy API
   // answers 1 for kernels that allocate tensor memory; the persistent loop needs no co-residency, so
   // a count above what fits only queues CTAs)
@@ -439,7 +439,7 @@ int launch_tc(const StageCommon &c, double ch, const double *term, const double 
       return -4;
     }
   }
-  constexpr int A = StageShape<N, float, float>::A;
+  constexpr int A = StageShape<N>::A;
   const int n_chunks = (c.u_end - c.u_begin + A - 1) / A;
   const int blocks_needed = (n_chunks + kTcWarps - 1) / kTcWarps;
   const int grid = std::max(1, std::min(blocks_needed, sched_ctas(per_sm, c.occ_pct) * sm_count));

@@ -114,7 +114,7 @@ void reschedule_cached(heom_run *r) {
 
 // The schedule of each part of a new run: the cache, else the tuner (if on), else the default.
 int schedule_new_run(heom_run *r) {
-  if (r->gen) return HEOM_OK;  // the general kernel keeps the default schedule
+  if (r->gen) return HEOM_OK;  // general runs keep the default schedule
   const int reps = g_autotune.load();
   for (int part = 0; part < (r->precision == HEOM_FP64 ? 1 : 2); ++part) {
     heom_schedule s{100, 1};
@@ -149,7 +149,7 @@ extern "C" int heom_tune(heom_run *r, int part, int reps, heom_schedule *tried, 
     return HEOM_E_ARG;
   }
   if (r->gen) {
-    set_error("heom_tune: runs on the general stage kernel keep the default schedule");
+    set_error("heom_tune: general runs (bath mask, laser field or more than 24 states) keep the default schedule");
     return HEOM_E_STATE;
   }
   std::vector<heom_schedule> t;
