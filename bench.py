@@ -22,6 +22,7 @@ import statistics
 import subprocess
 import sys
 import time
+from math import comb
 
 import numpy as np
 
@@ -44,17 +45,28 @@ def _peaks():
         return 6800.0, "fallback"
 
 
-# GB300 issues 2 FP64 FMAs (4 flops) per clock per SM: the nominal 1.25 TFLOP/s at the 2.07 GHz
-# maximum SM clock over 152 SMs; a dependent-FMA probe on this GPU gave 1.199 TFLOP/s at ~1.97 GHz.
-FP64_FLOPS_PER_CLK_SM = 4.0
-FP64_PEAK_TFLOPS = 1.2  # fallback when no SM clock was sampled
+# Issue rates measured on this GPU by chains of independent instructions: an FP64 instruction takes 18.7 clocks per
+# warp and SM (1.71 FMAs per clock), and 1.92 warp instructions of 32 x 32 + 64 bit integer multiply-add issue per clock and SM.
+FP64_CLK_PER_WARP_INSTR = 18.7
+INT_MAD_PER_CLK = 1.92
+FALLBACK_SM_MHZ = 1900.0
 
 
-def fp64_peak_tflops(sm_mhz, n_sm=152):
-    """FP64 ALU peak at the SM clock the leg ran at (nvidia-smi median under load)."""
-    if not sm_mhz:
-        return FP64_PEAK_TFLOPS, "fallback 1.2 TFLOP/s (no clock sample)"
-    return n_sm * FP64_FLOPS_PER_CLK_SM * sm_mhz * 1e6 / 1e12, f"{n_sm} SMs x 4 flop/clk x {sm_mhz:.0f} MHz"
+def fp64_roofline(avg_ms, fp64_instr, int_mads, alg_bytes, sm_mhz, n_sm, hbm_gbs):
+    """Roofline of an FP64 stage launch whose commutator runs in integers: the warp instructions that the algorithm needs
+    on the FP64 pipe and as integer multiply-adds, at the measured issue rates and the SM clock of the leg, and its
+    bytes at the copy bandwidth.  The slowest of the three is the bound."""
+    mhz = sm_mhz or FALLBACK_SM_MHZ
+    rate = n_sm * mhz * 1e6
+    ms = {"fp64_pipe": fp64_instr * FP64_CLK_PER_WARP_INSTR / rate * 1e3, "integer_multiply_add": int_mads / INT_MAD_PER_CLK / rate * 1e3,
+          "hbm": alg_bytes / (hbm_gbs * 1e9) * 1e3}
+    top = max(ms, key=ms.get)
+    work, unit = {"fp64_pipe": (fp64_instr / 1e9, "G FP64 warp instructions/s"),
+                  "integer_multiply_add": (int_mads / 1e9, "G integer multiply-add warp instructions/s"),
+                  "hbm": (alg_bytes / 1e9, "GB/s")}[top]
+    return {"bound": "hbm" if top == "hbm" else "alu", "achieved": work / (avg_ms / 1e3) if avg_ms > 0 else 0.0, "peak": work / (ms[top] / 1e3),
+            "unit": unit, "frac": ms[top] / avg_ms if avg_ms > 0 else 0.0, "bounds_ms": ms,
+            "peak_basis": f"{n_sm} SMs at {mhz:.0f} MHz" + ("" if sm_mhz else " (no clock sample)")}
 
 
 def _traffic():
@@ -203,8 +215,6 @@ def time_states(steps, warmup, ws, states=(14, 17, 19, 20, 22, 24), max_ados=2.5
     copy larger than L2).  Per size: ADO-RHS evals/s, the body launch time and its bandwidth on the
     per-unit count (4 tile transfers of N^2 FP32 complex elements + 2 M link-table entries per
     evaluation)."""
-    from math import comb
-
     from paper_1803_03498_gb300 import workloads as wl
 
     rows = []
@@ -269,16 +279,17 @@ def fp64_and_gate(prop, gate_steps, warmup, ws, clocks):
     assert obs64.shape == obs32.shape == (gate_steps + 1, N + 5)
     pop_err = float(np.max(np.abs(obs32[:, :N] - obs64[:, :N])))
     avg = kt["ms"] / max(kt["launches"], 1)
-    ach = kt["alg_flops"] / (kt["ms"] / 1000.0) / 1e12 if kt["ms"] > 0 else 0.0
     n_sm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    peak, basis = fp64_peak_tflops(clk["sm_mhz"] if clk else None, n_sm)
-    leg = {"value": _job_value(ws, n_ado, timed, ms), "unit": UNIT, "ms_per_step": ms / timed, "steps": timed,
-           "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                        "peak_basis": basis,
-                        "flops": "4 N^3 per ADO (Hermitian form: H s only, s H = (H s)^dagger) + 8 N^2 "
-                                 "+ 8 (N-1) per up link + 8 (2N-1) per down link",
-                        "kernel": "stage_col_kernel<14> (column form, FP64; the commutator runs in exact integers, so the "
-                                  "FP64 pipe's peak does not bound these flops)", "avg_launch_ms": avg, "schedule": sched},
+    # per ADO: 2 N columns of N sums of N products of six limb products; per column lane and row 2 conversion additions and
+    # the decay, per link record 2 FMAs on 2 N lanes, per pair of elements 2 additions and 2 FMAs
+    M, D = prop.system.n_modes, prop.system.D
+    recs = 2.0 * M * comb(M + D - 1, D - 1)
+    mads = n_ado * 2.0 * N * N * N * 6 / 32
+    fp64_instr = n_ado * (2.0 * N * N * 3 / 32 + 4.0 * -(-N * (N + 1) // 2 // 32)) + recs * 2.0
+    roof = fp64_roofline(avg, fp64_instr, mads, kt["alg_bytes"] / max(kt["launches"], 1), clk["sm_mhz"] if clk else None, n_sm, _peaks()[0])
+    roof.update({"kernel": "stage_col_kernel<14> (column form, FP64; the commutator in integers, three limbs)", "avg_launch_ms": avg,
+                 "schedule": sched})
+    leg = {"value": _job_value(ws, n_ado, timed, ms), "unit": UNIT, "ms_per_step": ms / timed, "steps": timed, "roofline": roof,
            "clocks": clk}
     gate = {"steps": gate_steps, "records": gate_steps + 1, "max_pop_err": pop_err, "bar": 1e-6,
             "pass": pop_err <= 1e-6,
@@ -372,8 +383,7 @@ def time_batch(steps=20, per_launch=10):
 def time_field(steps=40, warmup=3, sm_mhz=None):
     """Pump-pulse propagation of the FMO-like two-exciton space (7 sites: 29 states, K = 1, D = 4:
     3060 ADOs of 29 x 29) on the element kernels: classic four-copy RK4 with H(t) at each stage
-    time.  Device-timed steps; per-launch kernel time of the body launches; algorithmic flops per
-    ADO-RHS evaluation 16 N^3 (complex H(t)) + 8 N^2 + 8 per link record of each coupled state."""
+    time.  Device-timed steps; per-launch kernel time of the body launches."""
     import torch
 
     from paper_1803_03498_gb300 import heom
@@ -387,7 +397,6 @@ def time_field(steps=40, warmup=3, sm_mhz=None):
     per_state = s.bath_mask.sum(axis=1)  # states per bath's V
     K1 = s.K + 1
     recs = sum(int(np.sum(plus[:, l] >= 0) + np.sum(minus[:, l] >= 0)) * int(per_state[l // K1]) for l in range(s.n_modes))
-    flops_eval = n_ado * (16.0 * N ** 3 + 8.0 * N ** 2) + recs * 8.0 * N * 2
     out = {"workload": "fmo-like 7-site two-exciton space (29 states) K=1 D=4 (3060 ADOs), Gaussian pump "
                        "(60 cm^-1 peak coupling, sigma 15 fs), dt=0.5 fs, classic RK4 with H(t)",
            "unit": UNIT, "steps": steps}
@@ -409,12 +418,13 @@ def time_field(steps=40, warmup=3, sm_mhz=None):
         leg = {"value": n_ado * 4 * steps / (ms / 1000.0), "ms_per_step": ms / steps,
                "avg_launch_ms": kt["ms"] / max(kt["launches"], 1)}
         if precision == "fp64":
-            # body launches cover every ADO: one RHS evaluation each
-            ach = flops_eval / (leg["avg_launch_ms"] / 1000.0) / 1e12
+            # body launches cover every ADO: one RHS evaluation each.  Per pair of elements 8 N products (complex H) of six limb
+            # products; decay 3 FP64 instructions, two outputs 4, a link record 4 on the N + 1 pairs of its state
+            pairs = N * (N + 1) // 2
             n_sm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-            peak, basis = fp64_peak_tflops(sm_mhz, n_sm)
-            leg["roofline"] = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                               "frac": ach / peak, "peak_basis": basis, "kernel": "el_stage_kernel<double,double> (commutator in integers)"}
+            leg["roofline"] = fp64_roofline(leg["avg_launch_ms"], (n_ado * pairs * 7.0 + recs * (N + 1) * 4.0) / 32,
+                                            n_ado * pairs * 8.0 * N * 6 / 32, kt["alg_bytes"] / max(kt["launches"], 1), sm_mhz, n_sm, _peaks()[0])
+            leg["roofline"]["kernel"] = "el_stage_kernel<double,double> (commutator in integers)"
         out[precision] = leg
     return out
 
@@ -653,7 +663,7 @@ def main():
                          "alg_bytes": "per-unit figure: 4 N^2 x 8 B + 2 M x 4 B per ADO-RHS evaluation x the body ADOs",
                          "frac_horner": ach_horner / hbm_peak,
                          "alg_bytes_per_launch_horner": kt["alg_bytes"] / max(kt["launches"], 1),
-                         "kernel": "stage_kernel<14,float,float> (levels >= 2)",
+                         "kernel": "stage_kernel<14> (FP32 rows, levels >= 2)",
                          "peak_source": peak_src, "timed_launches": kt["launches"], "avg_launch_ms": avg_ms,
                          "schedule": kt["schedule"]},
             "split_tf32": {"value": v_tc, "unit": UNIT, "steps": tc_steps, "ms_per_step": ms_tc / tc_steps,
