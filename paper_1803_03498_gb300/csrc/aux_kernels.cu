@@ -41,8 +41,10 @@ __global__ void scatter_kernel(StateView dst, int Ep, int u_split, int body_fp32
   }
 }
 
+// status (or nullptr): takes the run's error word err, so that a small read is one copy.
 __global__ void gather_kernel(StateView src, int Ep, int u_split, int body_fp32, int vec, int n, int64_t u0, int64_t count,
-                              double *re, double *im) {
+                              double *re, double *im, const int *err, double *status) {
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = *err;
   const int64_t E = (int64_t)n * n;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count * E; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = t / E, e = t - c * E;

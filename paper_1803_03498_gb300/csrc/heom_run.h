@@ -27,7 +27,7 @@ __global__ void record_kernel(StateView y, int u_split, int body_fp32, int vec, 
 __global__ void scatter_kernel(StateView dst, int Ep, int u_split, int body_fp32, int vec, int n, int64_t u0, int64_t count,
                                const double *re, const double *im);
 __global__ void gather_kernel(StateView src, int Ep, int u_split, int body_fp32, int vec, int n, int64_t u0, int64_t count,
-                              double *re, double *im);
+                              double *re, double *im, const int *err, double *status);
 
 }  // namespace heom
 
@@ -106,7 +106,9 @@ namespace heom {
 // count check (graph capture: heom_batch_launch checks the counts per replay); the kernel keeps
 // the run's real max_records as its bound either way.
 int enqueue_record(heom_run *r, bool host_check = true);
+int status_error(int err_flag, const char *who);
 int device_status(heom_run *r, const char *who, int64_t *records);
+int read_range(heom_run *r, StateView state, int64_t u0, int64_t count, double *re, double *im, const char *who);
 int io_range(heom_run *r, StateView state, int64_t u0, int64_t count, double *re, double *im, bool to_device);
 
 // the RK4 driver (propagate.cu)

@@ -294,16 +294,7 @@ extern "C" int heom_propagate(heom_run *r, double dt_fs, int64_t n_steps, int64_
   return HEOM_OK;
 }
 
-// Waits for the run's stream and reads its device error word (and the number of records): every call that hands results
-// to the caller asks for it first.
-int heom::device_status(heom_run *r, const char *who, int64_t *records) {
-  int64_t cnt_err[2] = {0, 0};
-  cudaError_t e = cudaMemcpyAsync(cnt_err, r->rec_count, sizeof(cnt_err), cudaMemcpyDeviceToHost, r->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
-  if (e != cudaSuccess) return cuda_fail(who, e);
-  if (records) *records = cnt_err[0];
-  int err_flag = 0;
-  std::memcpy(&err_flag, &cnt_err[1], sizeof(int));
+int heom::status_error(int err_flag, const char *who) {
   if (err_flag & kErrBounds) {
     set_error(std::string(who) + ": a bounds check of the debug build failed (a link record names an ADO, state or "
               "record range outside the run; its results are invalid)");
@@ -315,6 +306,19 @@ int heom::device_status(heom_run *r, const char *who, int64_t *records) {
     return HEOM_E_TIMEOUT;
   }
   return HEOM_OK;
+}
+
+// Waits for the run's stream and reads its device error word (and the number of records): every call that hands results
+// to the caller asks for it first.
+int heom::device_status(heom_run *r, const char *who, int64_t *records) {
+  int64_t cnt_err[2] = {0, 0};
+  cudaError_t e = cudaMemcpyAsync(cnt_err, r->rec_count, sizeof(cnt_err), cudaMemcpyDeviceToHost, r->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
+  if (e != cudaSuccess) return cuda_fail(who, e);
+  if (records) *records = cnt_err[0];
+  int err_flag = 0;
+  std::memcpy(&err_flag, &cnt_err[1], sizeof(int));
+  return status_error(err_flag, who);
 }
 
 extern "C" int heom_observables(heom_run *r, double *out, int64_t cap_records, int64_t *written) {
@@ -345,6 +349,5 @@ extern "C" int heom_rhs_eval(heom_run *r, int64_t u0, int64_t count, double *re,
   if (r->has_field) field_g(r, r->t_fs);  // L at the current time
   int rc = run_stage(r, r->y, none, r->zA, 1.0);
   if (rc) return rc;
-  if ((rc = device_status(r, "heom_rhs_eval", nullptr))) return rc;
-  return io_range(r, r->zA, u0, count, re, im, false);
+  return read_range(r, r->zA, u0, count, re, im, "heom_rhs_eval");
 }
