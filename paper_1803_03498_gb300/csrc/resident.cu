@@ -302,6 +302,9 @@ ElShare share_of(const heom_run *r, int cap) {
   // the most CTAs each part can use: an element kernel splits an FP64 ADO down to 64 pairs
   const double max64 = (double)n64 * (run_lean(r) ? 1 : std::max(1, P / 64)), max32 = (double)nb;
   double w64 = std::min(std::max(1.0, a / kElGrain), max64), w32 = nb > 0 ? std::min(std::max(1.0, b / kElGrain), max32) : 0.0;
+  // a body taken by elements: a unit of 32 ADOs (the most that its records tell apart) for each CTA at the least, for a CTA builds
+  // the link ranges of every further unit again in every stage (2 states, 126 ADOs in one CTA 66 us per step, in four 32)
+  if (nb > 0 && !r->herm) w32 = std::max(w32, std::ceil((double)nb / 32));
   if (w64 + w32 > cap) {
     // a head keeps the CTAs that it can use, up to a quarter: an ADO of 17 to 22 states takes one about 10 us, so
     // two after each other in a CTA hold the body's CTAs at the barrier
