@@ -37,9 +37,9 @@ int fit_ados(int n, int pitch, int pairs, size_t real_bytes, bool general, size_
   return k;
 }
 
-template <typename CT, typename BT, bool CPLX>
+template <typename CT, typename BT, int FORM, bool CPLX>
 int launch_stage_kind(const ElStageArgs &a, const double *mup, cudaStream_t st, int sm_count) {
-  const auto kern = el_stage_kernel<CT, BT, sizeof(CT) == 8 ? kElFixed : kElGeneral, CPLX>;
+  const auto kern = el_stage_kernel<CT, BT, FORM, CPLX>;
   static std::atomic<bool> ready{false};
   if (!ready) {
     const int rc = max_smem((const void *)kern, "element stage kernel");
@@ -128,13 +128,21 @@ int launch_el_stage(int kind, const ElStageArgs &in, const double *mup, cudaStre
   a.apu = std::max(1, std::min(a.apu, n_ado / (2 * sm_count)));
   if (n_ado < 2 * sm_count) a.splits = std::max(1, std::min(2 * sm_count / n_ado, P / 64));
   const bool cplx = c.cplx_h || mup;
+  // Up to 4 states 4 n (8 n) FMAs are as fast as the splitting, whose steps follow each other (general runs of 4 states, 15 ADOs
+  // 38 us per step against 47; heads of complex mixed runs of 2 states 33.5 against 37).  Only runs that never
+  // take whole steps, so that both forms of launch of the others give the same bits.
+  const bool chain = c.n < 5 && (a.general || (kind == 2 && c.cplx_h));
+  auto go = [&](auto CT, auto BT, auto FORM) {
+    using C = decltype(CT);
+    using B = decltype(BT);
+    return cplx ? launch_stage_kind<C, B, FORM.value, true>(a, mup, st, sm_count) : launch_stage_kind<C, B, FORM.value, false>(a, mup, st, sm_count);
+  };
+  const std::integral_constant<int, kElFixed> fixed;
+  const std::integral_constant<int, kElGeneral> fma;
   switch (kind) {
-    case 0: return cplx ? launch_stage_kind<double, double, true>(a, mup, st, sm_count)
-                        : launch_stage_kind<double, double, false>(a, mup, st, sm_count);
-    case 1: return cplx ? launch_stage_kind<float, float, true>(a, mup, st, sm_count)
-                        : launch_stage_kind<float, float, false>(a, mup, st, sm_count);
-    default: return cplx ? launch_stage_kind<double, float, true>(a, mup, st, sm_count)
-                         : launch_stage_kind<double, float, false>(a, mup, st, sm_count);
+    case 0: return chain ? go(0.0, 0.0, fma) : go(0.0, 0.0, fixed);
+    case 1: return go(0.f, 0.f, fma);
+    default: return chain ? go(0.0, 0.f, fma) : go(0.0, 0.f, fixed);
   }
 }
 
