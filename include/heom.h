@@ -38,7 +38,10 @@ extern "C" {
                                 record naming an ADO, a state or a record range outside the run */
 
 /* Arithmetic of a run. */
-#define HEOM_FP64 0       /* every ADO stored and computed in FP64 */
+#define HEOM_FP64 0       /* every ADO stored and computed in FP64.  The commutator of most sizes is summed in
+                             integers of 90 bits from operands cut 84 bits below the largest element of their
+                             tile or column; a sum so weak that this would be less than an FP64 chain
+                             gives (below 2^-28 of the largest product) is taken from FP64 FMAs */
 #define HEOM_FP32_MIXED 1 /* levels >= 2 stored and computed in FP32; levels 0 and 1 (the root ADO
                              sigma_0 and its direct neighbours), the RK4 combination of sigma_0 and
                              every observable reduction in FP64 */
@@ -316,9 +319,9 @@ int heom_batch_destroy(heom_batch *b);
  * a real H, no laser field, at most 200,000 ADOs) of equal n_states advance in work-list launches:
  * one launch per RK4 stage and part (FP64 head, FP32 body) covers every such run of that size, each
  * run's stage arguments staged from its own workspace, so many small requests cost a few launches
- * per step instead of eight each.  Small FP64 runs share launches of many steps (as heom_propagate), ahead of
+ * per step instead of eight each.  Small FP64 runs share launches of many steps (as heom_propagate), beside
  * the others.  Other runs launch on their own, on the same stream.  Everything is
- * enqueued on cuda_stream (the launches of different sizes on library-created streams forked from and
+ * enqueued on cuda_stream (the launches of different sizes and kinds on library-created streams forked from and
  * joined back into it, with its priority), ordered after work already enqueued on each run's stream, and later work
  * on each run's stream is ordered after it; the call does not block, except that writing a run's
  * work-list stage arguments (its first grouped call, or a new dt_fs) waits for cuda_stream.
